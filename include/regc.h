@@ -464,8 +464,8 @@ REGC_API regc_status regc_counters(regc_handle *h, int64_t *moves, int64_t *exch
 
 /* Warps that evaluate a walker's moves in the plain sweep (1, 2 or 4; moves
  * evaluated speculatively per round and committed in order, so the chain does
- * not depend on it).  Chosen at creation from the replicas per SM (4 up to two
- * per SM, 2 up to four, else 1) unless the environment variable
+ * not depend on it).  Chosen at creation from the replicas per SM (4 up to 3.5
+ * per SM, 2 up to five, else 1) unless the environment variable
  * REGC_WARPS_PER_WALKER sets it; halved while one walker's shared memory
  * would not fit.  Delayed acceptance and the cluster species use one. */
 REGC_API regc_status regc_warps_per_walker(const regc_handle *h, int *warps);

@@ -20,8 +20,10 @@ LIB = os.path.join(BUILD, "libregc.so")
 # measurement tooling (the FP32 peak probe), kept out of the library proper
 PROBE_LIB = os.path.join(BUILD, "libregc_probe.so")
 PROBE_SOURCES = ["probe.cu"]
-SOURCES = ["sweep.cu", "exchange.cu", "mbar.cu", "regc_api.cu", "mbar_static.cu", "surrogate.cu", "walkers.cu", "batch.cu", "md.cu", "structure.cu"]
-HEADERS = ["regc_internal.cuh", "launch.h", "mbar.h", "surrogate.cuh", "handle.h", "cells.cuh"]
+SOURCES = ["sweep.cu", "sweep_species.cu", "batch_sweep.cu", "energy.cu", "exchange.cu", "mbar.cu", "regc_api.cu",
+           "mbar_static.cu", "surrogate.cu", "walkers.cu", "batch.cu", "md.cu", "structure.cu"]
+HEADERS = ["regc_internal.cuh", "launch.h", "mbar.h", "surrogate.cuh", "handle.h", "cells.cuh",
+           "walker.cuh", "sweep_launch.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "--ptxas-options=-v" if os.environ.get("REGC_PTXAS_VERBOSE") else "-w"]

@@ -3,7 +3,7 @@
 // A batch groups existing handles, each its own system (surface, box, grid,
 // Nmax).  Their walkers are sorted into size classes by Nmax; each class runs
 // as one persistent kernel whose warps take (system, walker) items from a
-// queue, largest systems first (csrc/sweep.cu: batch_sweep_kernel).  The
+// queue, largest systems first (csrc/batch_sweep.cu: batch_sweep_kernel).  The
 // classes run concurrently as parallel branches of one CUDA graph, followed by
 // one exchange attempt on every system's grid; the Philox counters advance on
 // the device, so the captured step replays without host work.  The shape of
@@ -27,8 +27,7 @@ constexpr size_t kMaxSmem = 232448;  // 227 KB per block on sm_103a
 
 struct Bucket {
     int nmax = 0;
-    bool da = false;                // its systems sample with delayed acceptance
-    bool cl = false;                // its systems carry a cluster species
+    BatchClass c{};                 // what its systems have in common
     int region = 0;                 // dynamic shared memory per walker (bytes) at k warps per walker
     int k = 1;                      // warps per walker
     std::vector<int2> items;        // (system, walker), largest systems first
@@ -140,7 +139,7 @@ cudaError_t record_step(regc_batch* b, std::vector<double>* ms_out) {
         for (int k = 0; k < nb && e == cudaSuccess; ++k) {
             const Bucket& q = b->buckets[k];
             e = launch_batch_sweep(b->d_sys, q.d_items, (int)q.items.size(), b->d_counters + k, q.wpc, q.k,
-                                   q.grid, q.region, q.da, q.cl, b->stream);
+                                   q.grid, q.region, q.c, b->stream);
             if (e == cudaSuccess) e = cudaEventRecord(ev[k + 1], b->stream);
         }
         if (e == cudaSuccess)
@@ -163,7 +162,7 @@ cudaError_t record_step(regc_batch* b, std::vector<double>* ms_out) {
         if (k > 0) e = cudaStreamWaitEvent(s, b->fork, 0);
         if (e == cudaSuccess)
             e = launch_batch_sweep(b->d_sys, q.d_items, (int)q.items.size(), b->d_counters + k, q.wpc, q.k,
-                                   q.grid, q.region, q.da, q.cl, s);
+                                   q.grid, q.region, q.c, s);
         if (e == cudaSuccess && k > 0) e = cudaEventRecord(b->join[k], s);
     }
     for (int k = 1; k < nb && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(b->stream, b->join[k], 0);
@@ -265,14 +264,14 @@ regc_status regc_batch_create(regc_handle* const* handles, int count, int sweeps
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
     // size classes by (Nmax, sampling mode, cluster); within a class the largest systems first
-    std::map<std::tuple<int, int, int>, std::vector<int>> by_nmax;
+    std::map<std::tuple<int, int, int, int>, std::vector<int>> by_nmax;
     for (int m = 0; m < count; ++m)
-        by_nmax[{handles[m]->nmax, b->member_da[m], handles[m]->P.n_cluster > 0 ? 1 : 0}].push_back(m);
+        by_nmax[{handles[m]->nmax, b->member_da[m], handles[m]->P.n_cluster > 0 ? 1 : 0,
+                 sweep_direct(handles[m]->P) ? 1 : 0}].push_back(m);
     for (auto it = by_nmax.rbegin(); it != by_nmax.rend(); ++it) {
         Bucket q;
         q.nmax = std::get<0>(it->first);
-        q.da = std::get<1>(it->first) != 0;
-        q.cl = std::get<2>(it->first) != 0;
+        q.c = BatchClass{std::get<1>(it->first) != 0, std::get<2>(it->first) != 0, std::get<3>(it->first) != 0};
         std::vector<int> ms = it->second;
         q.members = ms;
         std::stable_sort(ms.begin(), ms.end(), [&](int a, int c) {
@@ -289,18 +288,15 @@ regc_status regc_batch_create(regc_handle* const* handles, int count, int sweeps
     // per SM
     for (auto& q : b->buckets) {
         int best = 0;
-        const size_t stat = batch_static_smem(q.da);
+        const size_t stat = batch_static_smem(q.c.da);
         for (int k = 1; k <= 4 && e == cudaSuccess; k *= 2) {
-            if (k > 1 && (q.da || q.cl)) break;
+            if (k > 1 && (q.c.da || q.c.cl)) break;
             size_t region = 0;
-            for (int m : q.members) {
-                const regc_handle* h = handles[m];
-                region = std::max(region, sweep_smem_per_walker(h->nmax, h->P.cg.ncell, h->P.cg.cap, k));
-            }
+            for (int m : q.members) region = std::max(region, sweep_smem(handles[m]->P, k));
             region = (region + 15) / 16 * 16;
-            for (int wpc = 1; k * wpc <= batch_max_warps(q.da) && e == cudaSuccess; wpc *= 2) {
+            for (int wpc = 1; k * wpc <= batch_max_warps(q.c.da) && e == cudaSuccess; wpc *= 2) {
                 if ((size_t)wpc * region + stat > kMaxSmem) break;
-                const int occ = batch_occupancy(wpc, k, (int)region, q.da, q.cl);
+                const int occ = batch_occupancy(wpc, k, (int)region, q.c);
                 if (occ < 1) break;
                 q.cand.push_back({k, wpc, (int)region});
                 if (k == 1 && wpc * occ > best) {
@@ -312,7 +308,7 @@ regc_status regc_batch_create(regc_handle* const* handles, int count, int sweeps
             }
         }
         if (q.cand.empty()) e = cudaErrorInvalidValue;   // one walker does not fit
-        const int occ = batch_occupancy(q.wpc, q.k, q.region, q.da, q.cl);
+        const int occ = batch_occupancy(q.wpc, q.k, q.region, q.c);
         const int need = (int)((q.items.size() + q.wpc - 1) / q.wpc);
         q.grid = std::max(1, std::min(need, b->sms * std::max(occ, 1)));
     }
@@ -394,7 +390,7 @@ regc_status regc_batch_autotune(regc_batch* b, int rounds) {
         for (size_t c = 0; c < n_cand; ++c) {
             for (auto& q : b->buckets) {
                 const Bucket::Shape sh = q.cand[std::min(c, q.cand.size() - 1)];
-                const int occ = batch_occupancy(sh.wpc, sh.k, sh.region, q.da, q.cl);
+                const int occ = batch_occupancy(sh.wpc, sh.k, sh.region, q.c);
                 const int need = (int)((q.items.size() + sh.wpc - 1) / sh.wpc);
                 q.k = sh.k;
                 q.wpc = sh.wpc;

@@ -1,0 +1,153 @@
+// batch_sweep.cu -- the persistent sweep of a batch of uneven systems (sm_103a).
+// See walker.cuh.
+#include "walker.cuh"
+
+namespace regc {
+namespace {
+
+// Persistent sweep of a batch of walkers from several systems.  Every group
+// of K warps of the CTA is one walker at a time: its first thread takes the
+// next (system, walker) item from the queue, the group copies that system's
+// parameters into its slot of shared memory and runs the walker's sweeps in
+// its own shared-memory region of `region` bytes (K > 1: the speculative
+// walker, synchronised by the group's named barrier 1 + group); items are
+// listed largest first, so the queue balances the uneven costs.  DA: the
+// systems of the launch sample with delayed acceptance (their networks'
+// fragments take ~240 registers per thread, so at most kBatchMaxWarpsDA
+// walkers per CTA); CL: every system of the launch carries a cluster species;
+// DIRECT: its walkers enumerate all particles instead of a cell list.
+constexpr int kBatchMaxWarps = 16;
+constexpr int kBatchMaxWarpsDA = 4;
+
+template <bool DA, bool CL, bool DIRECT, int K>
+__global__ void __launch_bounds__(32 * (DA ? kBatchMaxWarpsDA : kBatchMaxWarps))
+    batch_sweep_kernel(const SweepParams* __restrict__ sys, const int2* __restrict__ items, int n_items,
+                       int* counter, int region) {
+    constexpr int kGroups = (DA ? kBatchMaxWarpsDA : kBatchMaxWarps) / K;
+    extern __shared__ __align__(16) char smem[];
+    __shared__ SweepParams Psh[kGroups];
+    __shared__ int item_sh[kGroups];
+    const int tid = threadIdx.x % (32 * K), grp = threadIdx.x / (32 * K);
+    const int bar = K == 1 ? 0 : 1 + grp;
+    char* mine = smem + (size_t)grp * region;
+    for (;;) {
+        int item = 0;
+        if (K == 1) {
+            if (tid == 0) item = atomicAdd(counter, 1);
+            item = __shfl_sync(FULL, item, 0);
+        } else {
+            if (tid == 0) item_sh[grp] = atomicAdd(counter, 1);
+            group_sync<K>(bar);
+            item = item_sh[grp];
+        }
+        if (item >= n_items) break;
+        const int2 mw = items[item];
+        const int* src = reinterpret_cast<const int*>(sys + mw.x);
+        int* dst = reinterpret_cast<int*>(&Psh[grp]);
+        for (int k = tid; k < (int)(sizeof(SweepParams) / sizeof(int)); k += 32 * K) dst[k] = src[k];
+        group_sync<K>(bar);
+        walker_sweep<K, false, DA, CL, DIRECT>(Psh[grp], mw.y, mine, tid, bar);
+        group_sync<K>(bar);   // the slot and the item are rewritten for the next walker
+    }
+}
+
+}  // namespace
+
+size_t batch_static_smem(bool da) {
+    return (sizeof(SweepParams) + sizeof(int)) * (da ? kBatchMaxWarpsDA : kBatchMaxWarps);
+}
+
+int batch_max_warps(bool da) { return da ? kBatchMaxWarpsDA : kBatchMaxWarps; }
+
+namespace {
+
+struct Launch {
+    const SweepParams* sys;
+    const int2* items;
+    int n_items;
+    int* counter;
+    int walkers_per_cta, grid, region;
+    cudaStream_t s;
+    cudaError_t err = cudaErrorInvalidValue;
+    template <bool DA, bool CL, bool DIRECT, int K>
+    void run() {
+        const size_t smem = (size_t)walkers_per_cta * region;
+        batch_sweep_kernel<DA, CL, DIRECT, K>
+            <<<grid, 32 * K * walkers_per_cta, smem, s>>>(sys, items, n_items, counter, region);
+        err = cudaGetLastError();
+    }
+};
+
+struct Prepare {
+    int max_smem;
+    cudaError_t err = cudaSuccess;
+    template <bool DA, bool CL, bool DIRECT, int K>
+    void run() {
+        if (err == cudaSuccess)
+            err = cudaFuncSetAttribute(batch_sweep_kernel<DA, CL, DIRECT, K>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       max_smem - (int)batch_static_smem(DA));
+    }
+};
+
+struct Occupancy {
+    int walkers_per_cta;
+    size_t smem;
+    int n = 0;
+    template <bool DA, bool CL, bool DIRECT, int K>
+    void run() {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_sweep_kernel<DA, CL, DIRECT, K>,
+                                                          32 * K * walkers_per_cta, smem) != cudaSuccess)
+            n = 0;
+    }
+};
+
+// f.run<DA, CL, DIRECT, K>() of a class; false where there is no such kernel:
+// delayed acceptance follows the cell list, and more than one warp per walker
+// is for plain one-species walkers.
+template <class F>
+bool dispatch(const BatchClass& c, int K, F& f) {
+    if (c.da && c.direct) return false;
+    if (K == 1) {
+        if (c.da && c.cl) f.template run<true, true, false, 1>();
+        else if (c.da) f.template run<true, false, false, 1>();
+        else if (c.cl && c.direct) f.template run<false, true, true, 1>();
+        else if (c.cl) f.template run<false, true, false, 1>();
+        else if (c.direct) f.template run<false, false, true, 1>();
+        else f.template run<false, false, false, 1>();
+        return true;
+    }
+    if (c.da || c.cl || (K != 2 && K != 4)) return false;
+    if (K == 2 && c.direct) f.template run<false, false, true, 2>();
+    else if (K == 2) f.template run<false, false, false, 2>();
+    else if (c.direct) f.template run<false, false, true, 4>();
+    else f.template run<false, false, false, 4>();
+    return true;
+}
+
+}  // namespace
+
+cudaError_t launch_batch_sweep(const SweepParams* sys, const int2* items, int n_items, int* counter,
+                               int walkers_per_cta, int warps_per_walker, int grid, int region, BatchClass c,
+                               cudaStream_t s) {
+    if (n_items <= 0) return cudaSuccess;
+    if (walkers_per_cta < 1 || warps_per_walker * walkers_per_cta > batch_max_warps(c.da) || grid < 1)
+        return cudaErrorInvalidValue;
+    Launch f{sys, items, n_items, counter, walkers_per_cta, grid, region, s};
+    if (!dispatch(c, warps_per_walker, f)) return cudaErrorInvalidValue;
+    return f.err;
+}
+
+cudaError_t batch_prepare(int max_smem) {
+    Prepare f{max_smem};
+    for (int bits = 0; bits < 8; ++bits)
+        for (int K = 1; K <= 4; K *= 2) dispatch(BatchClass{(bits & 1) != 0, (bits & 2) != 0, (bits & 4) != 0}, K, f);
+    return f.err;
+}
+
+int batch_occupancy(int walkers_per_cta, int warps_per_walker, int region, BatchClass c) {
+    Occupancy f{walkers_per_cta, (size_t)walkers_per_cta * region};   // within the limit batch_prepare set
+    return dispatch(c, warps_per_walker, f) ? f.n : 0;
+}
+
+}  // namespace regc

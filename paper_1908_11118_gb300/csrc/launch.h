@@ -7,12 +7,42 @@
 
 namespace regc {
 
-// Shared-memory bytes of the sweep kernel's CTA (one walker, W warps).
-size_t sweep_smem_per_walker(int nmax, int ncell, int cap, int warps_per_walker);
+// Nmax up to which a walker's moves enumerate every particle (walker.cuh).  A
+// stencil of 27 of the ncell cells spares the share 1 - 27 / ncell of the
+// distances and costs what about 52 of them do; with many walkers per SM the
+// smaller region counts too (more of them resident), and the line lies higher.
+// Microseconds of a ten-sweep launch, direct / cells, every walker nearly full:
+//   fcc(111), 168 cells, 16 walkers:   137 / 157 at Nmax 32, 158 / 158 at 64, 172 / 161 at 96
+//   periodic cube, 125 cells, 16 walkers:   167 / 192 at 20, 236 / 200 at 68
+//   periodic cube, 4096 walkers (27 per SM):   391 / 493 at 20, 578 / 640 at 68,
+//     652 / 683 at 128, 729 / 747 at 160, 809 / 782 at 192
+//   A18, 40 cells, 160 walkers of 20 particles:   88 / 105
+constexpr int kDirectMax = 160;
+
+inline int direct_limit(int ncell, long long walkers, int sms) {
+    const int line = walkers > 12LL * sms ? kDirectMax : 52;
+    if (ncell <= 27) return kDirectMax;
+    const long long n = (long long)line * ncell / (ncell - 27);
+    return n < kDirectMax ? (int)n : kDirectMax;
+}
+
+// Whether the system's walkers enumerate all particles with their nearest
+// images (walker.cuh) instead of a cell list; delayed acceptance follows the
+// cell list.
+inline bool sweep_direct(const SweepParams& P) { return P.direct && !P.delayed; }
+
+// Shared-memory bytes of one walker of the sweep kernel with W warps.
+size_t sweep_smem(const SweepParams& P, int warps_per_walker);
+
+// The bytes by which handles are admitted (at most 227 KB; never less than
+// sweep_smem of the same sizes).
+size_t sweep_smem_admitted(int nmax, int ncell, int cap, int warps_per_walker);
 
 // P.n_sweeps sweeps of every walker with P.warps_per_walker warps per walker;
 // P.trace may be null.
 cudaError_t launch_sweep(const SweepParams& P, cudaStream_t s);
+// launch_sweep of the systems with two mobile species or delayed acceptance.
+cudaError_t launch_sweep_species(const SweepParams& P, cudaStream_t s);
 
 // From-scratch fixed-point energy of every walker into out[S]; a pair inside
 // the hard-core guard sets ERR_OVERLAP (check_overlap 1) or ERR_NUMERIC
@@ -35,15 +65,20 @@ cudaError_t unpack_walkers(const float4* pos, long long count, int nmax, const i
 size_t batch_static_smem(bool da);
 int batch_max_warps(bool da);
 
+// What the systems of one batch launch have in common: da, sampling with
+// delayed acceptance; cl, a cluster species; direct, sweep_direct.
+struct BatchClass {
+    bool da, cl, direct;
+};
+
 // Persistent sweep of items (system, walker) of the systems sys[] (device
 // table; every system's n_sweeps and t0 are read from it), taken in order from
 // the queue *counter (zero before the launch); walkers_per_cta walkers of
 // warps_per_walker warps each per CTA (1, 2 or 4; more than one for plain
 // one-species systems only), each with `region` bytes of dynamic shared
-// memory.  da: every system of the items samples with delayed acceptance; cl:
-// every system carries a cluster species.
+// memory.
 cudaError_t launch_batch_sweep(const SweepParams* sys, const int2* items, int n_items, int* counter,
-                               int walkers_per_cta, int warps_per_walker, int grid, int region, bool da, bool cl,
+                               int walkers_per_cta, int warps_per_walker, int grid, int region, BatchClass c,
                                cudaStream_t s);
 
 // Allow every batch sweep kernel up to max_smem bytes of shared memory in all
@@ -51,7 +86,7 @@ cudaError_t launch_batch_sweep(const SweepParams* sys, const int2* items, int n_
 cudaError_t batch_prepare(int max_smem);
 
 // Resident CTAs per SM of the batch sweep kernel for this shape (0 if none fit).
-int batch_occupancy(int walkers_per_cta, int warps_per_walker, int region, bool da, bool cl);
+int batch_occupancy(int walkers_per_cta, int warps_per_walker, int region, BatchClass c);
 
 // One exchange attempt of every system's grid (attempt numbers e_ctr[]), then
 // e_ctr[m] += 1 and sys[m].t0 += n_sweeps on the device.

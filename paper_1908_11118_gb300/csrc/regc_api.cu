@@ -192,30 +192,30 @@ regc_status init_grid(const regc_potential* pot, const regc_surface* surf, const
         !(grid->e_bin < 4294967296.0))
         return REGC_EINVAL;
     // warps per walker = moves evaluated speculatively per round (1, 2 or 4).
-    // With many walkers per SM one is best: on the 1024-replica fcc(111)
-    // workload two and four warps run at 0.58x and 0.44x of one (instruction
-    // fetch and the round barriers outweigh the kept evaluations).  With about
-    // one walker per SM the issue slots are idle and speculation pays: 160
-    // replicas of the LJ A18 system run 1.33x faster with four warps; at 256
-    // fcc(111) replicas (1.7 per SM) two warps gain 3 % and four lose 18 %.
+    // A round of K costs one evaluation and K commits in order, so it pays
+    // while the issue slots are idle.  Microseconds of a ten-sweep launch with
+    // 1 / 2 / 4 warps (SMs: 152):
+    //   fcc(111):  64 walkers 310 / 273 / 236, 256: 316 / 272 / 250,
+    //              512: 314 / 286 / 264, 1024: 338 / 333 / 463
+    //   A18:       160: 136 / 111 / 89, 640: 181 / 172 / 200
+    //   fcc(100):  256: 210 / 196 / 191, 4096: 458 / 784 / 1083
     // REGC_WARPS_PER_WALKER overrides the choice.
-    int W = 1;
+    int W = 1, sms = 0;
     {
-        int dev = 0, sms = 0;
+        int dev = 0;
         if (cudaGetDevice(&dev) == cudaSuccess &&
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) {
             const long long n_rep = (long long)grid->L * grid->M;
-            if (4 * n_rep <= 5LL * sms) W = 4;
-            else if (n_rep <= 2LL * sms) W = 2;
+            if (2 * n_rep <= 7LL * sms) W = 4;
+            else if (n_rep <= 5LL * sms) W = 2;
         }
     }
     if (const char* env = getenv("REGC_WARPS_PER_WALKER")) {
         const int v = atoi(env);
         if (v == 1 || v == 2 || v == 4) W = v;
     }
-    while (W > 1 && sweep_smem_per_walker(grid->nmax, cg.ncell, cg.cap, W) > kMaxSmem) W /= 2;
-    const size_t spw = sweep_smem_per_walker(grid->nmax, cg.ncell, cg.cap, W);
-    if (spw > kMaxSmem) return REGC_EINVAL;
+    while (W > 1 && sweep_smem_admitted(grid->nmax, cg.ncell, cg.cap, W) > kMaxSmem) W /= 2;
+    if (sweep_smem_admitted(grid->nmax, cg.ncell, cg.cap, W) > kMaxSmem) return REGC_EINVAL;
 
     regc_handle* h = new (std::nothrow) regc_handle;
     if (!h) return REGC_ENOMEM;
@@ -238,7 +238,6 @@ regc_status init_grid(const regc_potential* pot, const regc_surface* surf, const
     h->z_lo = surf->z_lo;
     h->z_hi = surf->z_hi;
     h->periodic_z = periodic_z;
-    h->smem_per_walker = spw;
     const int S = h->S;
 
     // ---- per-state constants of the acceptance rules
@@ -407,9 +406,14 @@ regc_status init_grid(const regc_potential* pot, const regc_surface* surf, const
     P.e_bin = grid->e_bin;
     P.e_lo_fix = llround(grid->e_lo * kFixPerUnit);
     P.e_bin_fix = llround(grid->e_bin * kFixPerUnit);
+    P.e_bin_magic = ~0ull / (unsigned long long)P.e_bin_fix;
     P.n_e_bins = grid->n_e_bins;
-    P.smem_per_walker = (int)spw;
     P.warps_per_walker = W;
+    // every particle is enumerated where there are few; in a sheared cell only
+    // where the nearest image in the cell frame is beyond doubt the one within
+    // rc (a period above 2 rc sqrt(1 + shear^2) by more than rounding)
+    P.direct = grid->nmax <= direct_limit(cg.ncell, S, std::max(sms, 1)) &&
+               (shear == 0.0 || (double)surf->Lx > 2 * rc * su * (1 + 1e-5));
 
     // ---- device memory
     regc_status st_ = REGC_OK;
@@ -459,6 +463,9 @@ regc_status init_grid(const regc_potential* pot, const regc_surface* surf, const
     st.atoms = d_colat;
     st.all = d_all;
     st.n_all = surf->n_atoms;
+    st.one_type = surf->n_atoms > 0 ? surf->type[0] : 0;
+    for (int a = 0; a < surf->n_atoms; ++a)
+        if (surf->type[a] != st.one_type) st.one_type = -1;
     P.st = st;
     P.beta = d_beta;
     P.c_ins = d_cins;
@@ -900,6 +907,7 @@ regc_status regc_set_state_windows(regc_handle* h, int n_bins, double e_bin, con
     long long* d_lo = reinterpret_cast<long long*>(static_cast<char*>(block) + hist_bytes);
     h->P.hE_lo_fix = d_lo;
     h->P.hE_bin_fix = bin_fix;
+    h->P.hE_bin_magic = ~0ull / (unsigned long long)bin_fix;
     h->P.hE_bins = n_bins;
     e = cudaMemsetAsync(block, 0, hist_bytes, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_lo, lo_fix.data(), S * 8, cudaMemcpyHostToDevice, h->stream);

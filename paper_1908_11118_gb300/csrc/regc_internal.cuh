@@ -107,6 +107,7 @@ struct SurfaceTab {
     float isx, isy;        // columns per unit length
     float z_reach;         // surface atoms are out of reach at z >= z_reach
     int stride;            // slots per column, a multiple of 32
+    int one_type;          // the atoms' type where they have one, else -1
     const float4* atoms;   // [nsx*nsy][stride] images listed per column: x, y, z
                            // of the image (shifted by -L where exact), w = bits:
                            // type (0-1), query shifted by -Lx (2), -Ly (3),
@@ -165,11 +166,13 @@ struct SweepParams {
     unsigned long long* e_out;    // [S]
     double e_lo, e_bin;
     long long e_lo_fix, e_bin_fix;  // E-histogram origin and bin width in units of 2^-30
+    unsigned long long e_bin_magic;  // floor((2^64 - 1) / e_bin_fix)
     int n_e_bins;
     unsigned long long* hE;       // [S][hE_bins + 2] per-state energy histograms, or null: bin 0
                                   //     below the state's window, k + 1 window bin k, hE_bins + 1 beyond
     const long long* hE_lo_fix;   // [S] window origins in units of 2^-30
     long long hE_bin_fix;         // window bin width in units of 2^-30
+    unsigned long long hE_bin_magic;  // floor((2^64 - 1) / hE_bin_fix)
     int hE_bins;
     long long* move_counts;       // [S][6]
     unsigned long long* pair_counts;  // [6] pairs in rc, candidates, rounds, evaluations,
@@ -183,8 +186,8 @@ struct SweepParams {
                                   //    (insertion or removal), moves 1 .. mps-1 are displacements
     int m_first;                  // first move of the launch (1: its first step began with a
                                   //    replica exchange, so its particle exchange is not attempted)
-    int smem_per_walker;          // bytes
     int warps_per_walker;         // 1, 2 or 4
+    int direct;                   // 1: few enough particles to enumerate them all (walker.cuh)
     int delayed;                  // 1: two-stage delayed acceptance with the surrogate
     SurrogateDev net;             // the surrogate (delayed acceptance)
 };
