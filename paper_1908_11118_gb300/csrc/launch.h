@@ -141,6 +141,15 @@ cudaError_t surrogate_step(const float* theta_in, const float* X, const float* y
                            float* partial, float* grad, float* loss, float* theta, float* m, float* v, int adam_t,
                            float lr, bool tensor_cores, cudaStream_t s);
 
+// Whether a mini-batch of this size trains in one cluster of CTAs, and `steps`
+// training steps (rows drawn as surrogate_batch_index draws them for steps
+// adam_t + 1 .., gradient and Adam as surrogate_step's on tensor cores, bit for
+// bit) of such a mini-batch in one launch; loss [steps]: sums of squared residuals.
+bool surrogate_train_fits(int batch);
+cudaError_t surrogate_train_steps(float* theta, float* m, float* v, const float* X, const float* y, int count,
+                                  int batch, int steps, int adam_t, float lr, uint32_t k0, uint32_t k1, float* loss,
+                                  cudaStream_t s);
+
 // Seeded initial parameters (normal weights of standard deviation
 // scale / sqrt(fan-in), zero biases) into theta[5313].
 cudaError_t surrogate_init(float* theta, float scale, uint32_t k0, uint32_t k1, cudaStream_t s);

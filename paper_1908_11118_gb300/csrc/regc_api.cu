@@ -1451,15 +1451,26 @@ regc_status regc_surrogate_train(regc_handle* h, int steps, int batch, float lr,
     if (steps == 0) return REGC_OK;
     int* d_idx = nullptr;
     float *d_part = nullptr, *d_loss = nullptr;
-    cudaError_t e = cudaMallocAsync(&d_idx, batch * sizeof(int), h->stream);
-    if (e == cudaSuccess) e = cudaMallocAsync(&d_part, surrogate_partial_floats(batch) * sizeof(float), h->stream);
-    if (e == cudaSuccess) e = cudaMallocAsync(&d_loss, steps * sizeof(float), h->stream);
-    for (int k = 0; k < steps && e == cudaSuccess; ++k) {
-        h->adam_t += 1;
-        e = surrogate_batch_index(d_idx, batch, h->ds_count, (uint32_t)h->adam_t, h->P.key0, h->P.key1, h->stream);
-        if (e == cudaSuccess)
-            e = surrogate_step(h->d_theta, h->d_X, h->d_y, d_idx, batch, d_part, nullptr, d_loss + k, h->d_theta,
-                               h->d_adam_m, h->d_adam_v, h->adam_t, lr, true, h->stream);
+    cudaError_t e = cudaMallocAsync(&d_loss, steps * sizeof(float), h->stream);
+    if (surrogate_train_fits(batch)) {
+        // all the steps of a launch by one cluster of CTAs; at most 4096 of them
+        // (tens of milliseconds) a launch
+        for (int k = 0; k < steps && e == cudaSuccess; k += 4096) {
+            const int n = std::min(4096, steps - k);
+            e = surrogate_train_steps(h->d_theta, h->d_adam_m, h->d_adam_v, h->d_X, h->d_y, h->ds_count, batch, n,
+                                      h->adam_t, lr, h->P.key0, h->P.key1, d_loss + k, h->stream);
+            if (e == cudaSuccess) h->adam_t += n;
+        }
+    } else {
+        if (e == cudaSuccess) e = cudaMallocAsync(&d_idx, batch * sizeof(int), h->stream);
+        if (e == cudaSuccess) e = cudaMallocAsync(&d_part, surrogate_partial_floats(batch) * sizeof(float), h->stream);
+        for (int k = 0; k < steps && e == cudaSuccess; ++k) {
+            h->adam_t += 1;
+            e = surrogate_batch_index(d_idx, batch, h->ds_count, (uint32_t)h->adam_t, h->P.key0, h->P.key1, h->stream);
+            if (e == cudaSuccess)
+                e = surrogate_step(h->d_theta, h->d_X, h->d_y, d_idx, batch, d_part, nullptr, d_loss + k, h->d_theta,
+                                   h->d_adam_m, h->d_adam_v, h->adam_t, lr, true, h->stream);
+        }
     }
     if (e == cudaSuccess) e = surrogate_pack(h->d_theta, h->sur, h->stream);
     std::vector<float> lsum(steps);

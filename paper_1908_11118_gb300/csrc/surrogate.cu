@@ -9,8 +9,12 @@
 //   * grad_kernel / reduce_adam_kernel: one step of mini-batch training -- the
 //     forward and backward passes of 128 rows per CTA in shared memory, the
 //     per-CTA gradients summed in a fixed order, and Adam on the FP32 masters.
+#include <cooperative_groups.h>
+
 #include "launch.h"
 #include "surrogate.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace regc {
 namespace {
@@ -278,7 +282,6 @@ __global__ void __launch_bounds__(kRows) grad_kernel(const float* theta, const f
     }
 }
 
-// Sum the per-CTA gradients in a fixed order; optionally take an Adam step.
 // ------------------------------------------------ training on tensor cores
 //
 // The same gradient as grad_kernel with every matrix product on BF16
@@ -299,10 +302,14 @@ constexpr int kTcWarps = 4;
 constexpr int kTcRows = 32 * kTcWarps;
 constexpr int kTcLd = kTcRows + 8;   // row stride (bf16) of the transposed tiles
 
+// Row strides of the weights (bf16): 12 and 36 words, so that the eight rows a
+// B fragment takes lie in different banks.
+constexpr int kTcLd1 = kNF + 8, kTcLd2 = kNH + 8;
+
 struct TcSmem {
-    __nv_bfloat16 w1u[kNH][kNF];       // W1 unit-major: [u][k]
-    __nv_bfloat16 w2u[kNH][kNH];       // W2 unit-major: [v][u] (forward B)
-    __nv_bfloat16 w2r[kNH][kNH];       // W2 as stored: [u][v] (backward B)
+    __nv_bfloat16 w1u[kNH][kTcLd1];    // W1 unit-major: [u][k]
+    __nv_bfloat16 w2u[kNH][kTcLd2];    // W2 unit-major: [v][u] (forward B)
+    __nv_bfloat16 w2r[kNH][kTcLd2];    // W2 as stored: [u][v] (backward B)
     float w3[kNH], b1[kNH], b2[kNH];
     float b3, pad[3];
     __nv_bfloat16 xt[kNF][kTcLd];      // bf(X)^T
@@ -326,63 +333,49 @@ __device__ __forceinline__ float sum_over_g(float v) {
     return v;
 }
 
-__global__ void __launch_bounds__(kTcRows) grad_tc_kernel(const float* theta, const float* X, const float* yv,
-                                                          const int* idx, int n, float scale, float* partial,
-                                                          float* partial_loss) {
-    extern __shared__ __align__(16) unsigned char tc_raw[];
-    TcSmem& sm = *reinterpret_cast<TcSmem*>(tc_raw);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int g = lane >> 2, t = lane & 3;
-    const float* W1 = theta;
-    const float* B1 = W1 + kNF * kNH;
-    const float* W2 = B1 + kNH;
-    const float* B2 = W2 + kNH * kNH;
-    const float* W3 = B2 + kNH;
-    for (int i = tid; i < kNH * kNH; i += kTcRows) {
-        const int u = i / kNH, v = i % kNH;   // W2[u][v]
-        const __nv_bfloat16 w = __float2bfloat16_rn(W2[i]);
-        sm.w2r[u][v] = w;
-        sm.w2u[v][u] = w;
-        if (i < kNF * kNH) {
-            const int k = i / kNH, uu = i % kNH;   // W1[k][uu]
-            sm.w1u[uu][k] = __float2bfloat16_rn(W1[i]);
-        }
-        if (i < kNH) {
-            sm.w3[i] = W3[i];
-            sm.b1[i] = B1[i];
-            sm.b2[i] = B2[i];
-        }
+// Write parameter i of the master vector into the operand copies.
+__device__ __forceinline__ void tc_store_param(TcSmem& sm, int i, float v) {
+    constexpr int o1 = kNF * kNH, o2 = o1 + kNH, o3 = o2 + kNH * kNH, o4 = o3 + kNH, o5 = o4 + kNH;
+    if (i < o1) {
+        sm.w1u[i % kNH][i / kNH] = __float2bfloat16_rn(v);   // W1[k][u]
+    } else if (i < o2) {
+        sm.b1[i - o1] = v;
+    } else if (i < o3) {
+        const int u = (i - o2) / kNH, q = (i - o2) % kNH;    // W2[u][q]
+        const __nv_bfloat16 w = __float2bfloat16_rn(v);
+        sm.w2r[u][q] = w;
+        sm.w2u[q][u] = w;
+    } else if (i < o4) {
+        sm.b2[i - o3] = v;
+    } else if (i < o5) {
+        sm.w3[i - o4] = v;
+    } else {
+        sm.b3 = v;
     }
-    if (tid == 0) sm.b3 = W3[kNH];
-    // layer-1 A fragments: this warp's rows 32 warp + 16 mt + (g, g + 8)
-    const int row0 = blockIdx.x * kTcRows + warp * 32;
-    uint32_t ax[2][4];
-    int src[2][2];
-    bool act[2][2];
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int row = row0 + 16 * mt + g + 8 * h;
-            act[mt][h] = row < n;
-            src[mt][h] = act[mt][h] ? (idx ? idx[row] : row) : 0;
-            float2 lo = make_float2(0.f, 0.f), hi = make_float2(0.f, 0.f);
-            if (act[mt][h]) {
-                const float* xr = X + size_t(src[mt][h]) * kNF;
-                lo = make_float2(xr[2 * t], xr[2 * t + 1]);
-                hi = make_float2(xr[2 * t + 8], xr[2 * t + 9]);
-            }
-            ax[mt][h] = pack_bf16(lo.x, lo.y);        // A regs 0 (row g) and 1 (row g + 8)
-            ax[mt][2 + h] = pack_bf16(hi.x, hi.y);    // A regs 2 and 3
-            const int r = warp * 32 + 16 * mt + g + 8 * h;   // row within the CTA
-            const __nv_bfloat162 l2 = *reinterpret_cast<const __nv_bfloat162*>(&ax[mt][h]);
-            const __nv_bfloat162 h2 = *reinterpret_cast<const __nv_bfloat162*>(&ax[mt][2 + h]);
-            sm.xt[2 * t][r] = l2.x;
-            sm.xt[2 * t + 1][r] = l2.y;
-            sm.xt[2 * t + 8][r] = h2.x;
-            sm.xt[2 * t + 9][r] = h2.y;
-        }
-    }
+}
+
+// Layer-1 A registers of one row (h = 0: row g, 1: row g + 8 of 16-row tile mt
+// of this warp) from its features 2t, 2t + 1 (lo) and 2t + 8, 2t + 9 (hi), and
+// the row's place in the transposed copy.
+__device__ __forceinline__ void tc_row(TcSmem& sm, uint32_t (&ax)[2][4], int mt, int h, float2 lo, float2 hi,
+                                       int warp, int g, int t) {
+    ax[mt][h] = pack_bf16(lo.x, lo.y);        // A regs 0 (row g) and 1 (row g + 8)
+    ax[mt][2 + h] = pack_bf16(hi.x, hi.y);    // A regs 2 and 3
+    const int r = warp * 32 + 16 * mt + g + 8 * h;   // row within the CTA
+    const __nv_bfloat162 l2 = *reinterpret_cast<const __nv_bfloat162*>(&ax[mt][h]);
+    const __nv_bfloat162 h2 = *reinterpret_cast<const __nv_bfloat162*>(&ax[mt][2 + h]);
+    sm.xt[2 * t][r] = l2.x;
+    sm.xt[2 * t + 1][r] = l2.y;
+    sm.xt[2 * t + 8][r] = h2.x;
+    sm.xt[2 * t + 9][r] = h2.y;
+}
+
+// Forward and backward pass of the CTA's rows from their layer-1 fragments ax
+// (act: the row exists; y: its target): this CTA's gradient into G [5313], its
+// sum of squared residuals into *loss.
+__device__ __forceinline__ void tc_gradient(TcSmem& sm, const uint32_t (&ax)[2][4], const bool (&act)[2][2],
+                                            const float (&y)[2][2], float scale, float* G, float* loss, int tid) {
+    const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
     __syncthreads();   // the weights in shared memory
     // forward, layer 1: z1 (kept for silu'), bf(h1) as layer-2 A fragments and transposed
     float z1[2][8][4];
@@ -455,7 +448,7 @@ __global__ void __launch_bounds__(kTcRows) grad_tc_kernel(const float* theta, co
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const float res = act[mt][h] ? e[mt][h] - yv[src[mt][h]] : 0.f;
+            const float res = act[mt][h] ? e[mt][h] - y[mt][h] : 0.f;
             ge[mt][h] = 2.0f * res * scale;
             if (t == 0) {
                 sq = fmaf(res, res, sq);
@@ -568,7 +561,6 @@ __global__ void __launch_bounds__(kTcRows) grad_tc_kernel(const float* theta, co
         sm.red_s[warp][1] = sq;
     }
     __syncthreads();   // every warp's transposed tiles and partial sums
-    float* G = partial + size_t(blockIdx.x) * kNParams;
     float* gW1 = G;
     float* gb1 = gW1 + kNF * kNH;
     float* gW2 = gb1 + kNH;
@@ -628,10 +620,509 @@ __global__ void __launch_bounds__(kTcRows) grad_tc_kernel(const float* theta, co
             b += sm.red_s[w][1];
         }
         gW3[kNH] = a;                 // db3
-        partial_loss[blockIdx.x] = b;
+        *loss = b;
     }
 }
 
+__global__ void __launch_bounds__(kTcRows) grad_tc_kernel(const float* theta, const float* X, const float* yv,
+                                                          const int* idx, int n, float scale, float* partial,
+                                                          float* partial_loss) {
+    extern __shared__ __align__(16) unsigned char tc_raw[];
+    TcSmem& sm = *reinterpret_cast<TcSmem*>(tc_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int g = lane >> 2, t = lane & 3;
+    for (int i = tid; i < kNParams; i += kTcRows) tc_store_param(sm, i, theta[i]);
+    // layer-1 A fragments: this warp's rows 32 warp + 16 mt + (g, g + 8)
+    const int row0 = blockIdx.x * kTcRows + warp * 32;
+    uint32_t ax[2][4];
+    float y[2][2];
+    bool act[2][2];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int row = row0 + 16 * mt + g + 8 * h;
+            act[mt][h] = row < n;
+            const int src = act[mt][h] ? (idx ? idx[row] : row) : 0;
+            float2 lo = make_float2(0.f, 0.f), hi = make_float2(0.f, 0.f);
+            y[mt][h] = 0.f;
+            if (act[mt][h]) {
+                const float* xr = X + size_t(src) * kNF;
+                lo = make_float2(xr[2 * t], xr[2 * t + 1]);
+                hi = make_float2(xr[2 * t + 8], xr[2 * t + 9]);
+                y[mt][h] = yv[src];
+            }
+            tc_row(sm, ax, mt, h, lo, hi, warp, g, t);
+        }
+    }
+    tc_gradient(sm, ax, act, y, scale, partial + size_t(blockIdx.x) * kNParams, partial_loss + blockIdx.x, tid);
+}
+
+// One Adam step of a parameter (t-th step: c1 = 1 - b1^t, c2 = 1 - b2^t).
+__device__ __forceinline__ void adam_update(float g, float c1, float c2, float lr, float& m, float& v, float& theta) {
+    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    const float mi = b1 * m + (1.f - b1) * g;
+    const float vi = b2 * v + (1.f - b2) * g * g;
+    m = mi;
+    v = vi;
+    const float mh = mi / c1;
+    const float vh = vi / c2;
+    theta -= lr * mh / (sqrtf(vh) + eps);
+}
+
+// Many training steps in one launch: a cluster of one CTA per 128 rows of the
+// mini-batch (at most eight), each with a copy of the operands in shared
+// memory.  Per step: the gradient of the CTA's rows into its shared memory; the
+// cluster meets; CTA r adds the CTAs' gradients of its share of the parameters
+// through distributed shared memory, in CTA order, takes their Adam step (the
+// FP32 masters and moments of its share stay in its shared memory) and writes
+// the new operands into every CTA's copy; the cluster meets again.  The rows of
+// the next step are drawn (Philox stream 6) and requested while this one runs.
+//
+// A step is one chain of dependent pieces, so what counts is its latency, and
+// what makes it up are the SiLUs and their derivatives of 128 x 128 units by
+// few warps.  Eight warps share them: warps w and w + 4 take the same 32 rows,
+// one the lower half of each layer's units, the other the upper, and pass each
+// other the A fragments (and the running output sum) through shared memory.
+// Every sum keeps the terms and the order it has in tc_gradient, hence its
+// bits.
+constexpr int kMaxTrainCtas = 8;   // the portable cluster size
+constexpr int kXLd = kNF + 4;      // padded row of the staged features
+constexpr int kTrainThreads = 2 * kTcRows;
+
+struct TrainSmem {
+    TcSmem tc;
+    float grad[kNParams + 3];
+    float loss, pad[3];
+    float x[2][kTcRows][kXLd];
+    float y[2][kTcRows];
+    uint32_t xch[kTcWarps][2][16][32];   // A fragments of the two halves' units, by pair of warps
+    float o[kTcWarps][4][32];            // running output sums of the lower halves
+    float e[kTcWarps][4][32];            // outputs
+    float own[1];              // [3][share]: theta, m, v of this CTA's share
+};
+
+// Barrier of the two warps of a pair.
+__device__ __forceinline__ void pair_sync(int pair) {
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + pair) : "memory");
+}
+
+// Write this half's A words into the pair's exchange and its transposed copy.
+__device__ __forceinline__ void share_frag(uint32_t (*xch)[32], __nv_bfloat16 (*tr)[kTcLd],
+                                           const uint32_t (&own)[2][2][4], int pair, int half, int lane) {
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int kh = 0; kh < 2; ++kh) {
+            const uint32_t(&r)[4] = own[mt][kh];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) xch[8 * mt + 4 * kh + q][lane] = r[q];
+            const int rg = pair * 32 + 16 * mt + g, u = 16 * (2 * half + kh) + 2 * t;
+            const __nv_bfloat162 a0 = *reinterpret_cast<const __nv_bfloat162*>(&r[0]);
+            const __nv_bfloat162 a1 = *reinterpret_cast<const __nv_bfloat162*>(&r[1]);
+            const __nv_bfloat162 a2 = *reinterpret_cast<const __nv_bfloat162*>(&r[2]);
+            const __nv_bfloat162 a3 = *reinterpret_cast<const __nv_bfloat162*>(&r[3]);
+            tr[u][rg] = a0.x;     tr[u + 1][rg] = a0.y;
+            tr[u][rg + 8] = a1.x; tr[u + 1][rg + 8] = a1.y;
+            tr[u + 8][rg] = a2.x; tr[u + 9][rg] = a2.y;
+            tr[u + 8][rg + 8] = a3.x; tr[u + 9][rg + 8] = a3.y;
+        }
+}
+
+// The A fragments of all units from this half's and the partner's.
+__device__ __forceinline__ void gather_frag(const uint32_t (*other)[32], const uint32_t (&own)[2][2][4], int half,
+                                            int lane, uint32_t (&a)[2][4][4]) {
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int kh = 0; kh < 2; ++kh)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t x = other[8 * mt + 4 * kh + q][lane];
+                a[mt][kh][q] = half ? x : own[mt][kh][q];
+                a[mt][2 + kh][q] = half ? own[mt][kh][q] : x;
+            }
+}
+
+// tc_gradient by eight warps: this CTA's gradient into sm.grad, its sum of
+// squared residuals into sm.loss.
+__device__ __forceinline__ void train_gradient(TrainSmem& ts, const uint32_t (&ax)[2][4], const bool (&act)[2][2],
+                                               const float (&y)[2][2], float scale, int tid) {
+    TcSmem& sm = ts.tc;
+    const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    const int pair = warp & 3, half = warp >> 2;
+    __syncthreads();   // the operands and the transposed rows
+    // forward, layer 1: this half's units 8 (4 half + jj) ..
+    float z1[2][4][4];
+    uint32_t own[2][2][4], a[2][4][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+            const int j = 4 * half + jj, u = 8 * j + 2 * t;
+            z1[mt][jj][0] = z1[mt][jj][2] = sm.b1[u];
+            z1[mt][jj][1] = z1[mt][jj][3] = sm.b1[u + 1];
+            const uint32_t b[2] = {lds_u32(&sm.w1u[8 * j + g][2 * t]), lds_u32(&sm.w1u[8 * j + g][2 * t + 8])};
+            mma_bf16(z1[mt][jj], ax[mt], b);
+        }
+#pragma unroll
+        for (int kh = 0; kh < 2; ++kh)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float* c = z1[mt][2 * kh + q];
+                own[mt][kh][2 * q] = pack_bf16(silu_f(c[0]), silu_f(c[1]));
+                own[mt][kh][2 * q + 1] = pack_bf16(silu_f(c[2]), silu_f(c[3]));
+            }
+    }
+    share_frag(ts.xch[pair][half], sm.h1t, own, pair, half, lane);
+    pair_sync(pair);
+    gather_frag(ts.xch[pair][half ^ 1], own, half, lane, a);
+    // forward, layer 2
+    float z2[2][4][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+            const int j = 4 * half + jj, v = 8 * j + 2 * t;
+            z2[mt][jj][0] = z2[mt][jj][2] = sm.b2[v];
+            z2[mt][jj][1] = z2[mt][jj][3] = sm.b2[v + 1];
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                const uint32_t b[2] = {lds_u32(&sm.w2u[8 * j + g][16 * kk + 2 * t]),
+                                       lds_u32(&sm.w2u[8 * j + g][16 * kk + 2 * t + 8])};
+                mma_bf16(z2[mt][jj], a[mt][kk], b);
+            }
+        }
+    // the output: the lower half's units first, then the upper's
+    float s2[2][4][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) s2[mt][jj][c] = silu_f(z2[mt][jj][c]);
+    float o[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, e[2][2];
+    if (half) {
+        pair_sync(pair);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) o[q >> 1][q & 1] = ts.o[pair][q][lane];
+    }
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+            const int v = 8 * (4 * half + jj) + 2 * t;
+            o[mt][0] = fmaf(s2[mt][jj][0], sm.w3[v], fmaf(s2[mt][jj][1], sm.w3[v + 1], o[mt][0]));
+            o[mt][1] = fmaf(s2[mt][jj][2], sm.w3[v], fmaf(s2[mt][jj][3], sm.w3[v + 1], o[mt][1]));
+        }
+    if (!half) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) ts.o[pair][q][lane] = o[q >> 1][q & 1];
+        pair_sync(pair);
+    }
+    // meanwhile: the derivatives
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) z2[mt][jj][c] = dsilu_f(z2[mt][jj][c]);
+    if (half) {
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                // the four lanes of a group hold the row's partial dot products
+                float x = o[mt][h];
+                x += __shfl_xor_sync(FULL, x, 1);
+                x += __shfl_xor_sync(FULL, x, 2);
+                e[mt][h] = x + sm.b3;
+                ts.e[pair][2 * mt + h][lane] = e[mt][h];
+            }
+    }
+    pair_sync(pair);
+    if (!half) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) e[q >> 1][q & 1] = ts.e[pair][q][lane];
+    }
+    // residuals and d loss / d e
+    float ge[2][2], sq = 0.f, gsum = 0.f;
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float res = act[mt][h] ? e[mt][h] - y[mt][h] : 0.f;
+            ge[mt][h] = 2.0f * res * scale;
+            if (t == 0) {
+                sq = fmaf(res, res, sq);
+                gsum += ge[mt][h];
+            }
+        }
+    // dW3, db2 partials and dz2
+    float dw3[4][2], db2[4][2];
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) dw3[jj][0] = dw3[jj][1] = db2[jj][0] = db2[jj][1] = 0.f;
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+            const int v = 8 * (4 * half + jj) + 2 * t;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float gr = ge[mt][c >> 1];
+                dw3[jj][c & 1] = fmaf(gr, s2[mt][jj][c], dw3[jj][c & 1]);
+                const float d = gr * sm.w3[v + (c & 1)] * z2[mt][jj][c];
+                z2[mt][jj][c] = d;
+                db2[jj][c & 1] += d;
+            }
+        }
+#pragma unroll
+        for (int kh = 0; kh < 2; ++kh)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float* c = z2[mt][2 * kh + q];
+                own[mt][kh][2 * q] = pack_bf16(c[0], c[1]);
+                own[mt][kh][2 * q + 1] = pack_bf16(c[2], c[3]);
+            }
+    }
+    share_frag(ts.xch[pair][half], sm.d2t, own, pair, half, lane);
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) z1[mt][jj][c] = dsilu_f(z1[mt][jj][c]);
+    pair_sync(pair);
+    gather_frag(ts.xch[pair][half ^ 1], own, half, lane, a);
+    // backward through layer 2
+    float db1[4][2];
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) db1[jj][0] = db1[jj][1] = 0.f;
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+            const int j = 4 * half + jj;
+            float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+                const uint32_t b[2] = {lds_u32(&sm.w2r[8 * j + g][16 * kk + 2 * t]),
+                                       lds_u32(&sm.w2r[8 * j + g][16 * kk + 2 * t + 8])};
+                mma_bf16(c, a[mt][kk], b);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float d = c[q] * z1[mt][jj][q];
+                z1[mt][jj][q] = d;
+                db1[jj][q & 1] += d;
+            }
+        }
+#pragma unroll
+        for (int kh = 0; kh < 2; ++kh)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const float* c = z1[mt][2 * kh + q];
+                own[mt][kh][2 * q] = pack_bf16(c[0], c[1]);
+                own[mt][kh][2 * q + 1] = pack_bf16(c[2], c[3]);
+            }
+    }
+    // (the exchange is read by the partner up to its own writes here, so the
+    // transposed copy alone is written)
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int kh = 0; kh < 2; ++kh) {
+            const uint32_t(&r)[4] = own[mt][kh];
+            const int rg = pair * 32 + 16 * mt + g, u = 16 * (2 * half + kh) + 2 * t;
+            const __nv_bfloat162 a0 = *reinterpret_cast<const __nv_bfloat162*>(&r[0]);
+            const __nv_bfloat162 a1 = *reinterpret_cast<const __nv_bfloat162*>(&r[1]);
+            const __nv_bfloat162 a2 = *reinterpret_cast<const __nv_bfloat162*>(&r[2]);
+            const __nv_bfloat162 a3 = *reinterpret_cast<const __nv_bfloat162*>(&r[3]);
+            sm.d1t[u][rg] = a0.x;     sm.d1t[u + 1][rg] = a0.y;
+            sm.d1t[u][rg + 8] = a1.x; sm.d1t[u + 1][rg + 8] = a1.y;
+            sm.d1t[u + 8][rg] = a2.x; sm.d1t[u + 9][rg] = a2.y;
+            sm.d1t[u + 8][rg + 8] = a3.x; sm.d1t[u + 9][rg + 8] = a3.y;
+        }
+    // per-warp sums over rows of dW3, db2, db1, db3 and the squared residuals
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const float s3 = sum_over_g(dw3[jj][q]), sb2 = sum_over_g(db2[jj][q]), sb1 = sum_over_g(db1[jj][q]);
+            if (g == 0) {
+                const int u = 8 * (4 * half + jj) + 2 * t + q;
+                sm.red[pair][0][u] = s3;
+                sm.red[pair][1][u] = sb2;
+                sm.red[pair][2][u] = sb1;
+            }
+        }
+    sq = sum_over_g(sq);
+    gsum = sum_over_g(gsum);
+    if (lane == 0 && !half) {
+        sm.red_s[pair][0] = gsum;
+        sm.red_s[pair][1] = sq;
+    }
+    __syncthreads();   // every warp's transposed tiles and partial sums
+    float* gW1 = ts.grad;
+    float* gb1 = gW1 + kNF * kNH;
+    float* gW2 = gb1 + kNH;
+    float* gb2 = gW2 + kNH * kNH;
+    float* gW3 = gb2 + kNH;
+    // dW2 = bf(h1)^T bf(dz2) over the CTA's rows: 4 x 8 tiles of 16 x 8, four per
+    // warp, the two of each step sharing their rows of bf(h1)
+#pragma unroll 1
+    for (int tile = 2 * warp; tile < 32; tile += 16) {
+        const int u0 = 16 * (tile >> 3), v0 = 8 * (tile & 7);
+        float c[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+        for (int kk = 0; kk < kTcRows / 16; ++kk) {
+            const int r = 16 * kk + 2 * t;
+            const uint32_t h[4] = {lds_u32(&sm.h1t[u0 + g][r]), lds_u32(&sm.h1t[u0 + g + 8][r]),
+                                   lds_u32(&sm.h1t[u0 + g][r + 8]), lds_u32(&sm.h1t[u0 + g + 8][r + 8])};
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const uint32_t b[2] = {lds_u32(&sm.d2t[v0 + 8 * q + g][r]), lds_u32(&sm.d2t[v0 + 8 * q + g][r + 8])};
+                mma_bf16(c[q], h, b);
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int v = v0 + 8 * q + 2 * t;
+            *reinterpret_cast<float2*>(&gW2[(u0 + g) * kNH + v]) = make_float2(c[q][0], c[q][1]);
+            *reinterpret_cast<float2*>(&gW2[(u0 + g + 8) * kNH + v]) = make_float2(c[q][2], c[q][3]);
+        }
+    }
+    // dW1 = bf(X)^T bf(dz1): 1 x 8 tiles, one per warp
+    {
+        const int u0 = 8 * warp;
+        float c[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int kk = 0; kk < kTcRows / 16; ++kk) {
+            const int r = 16 * kk + 2 * t;
+            const uint32_t x[4] = {lds_u32(&sm.xt[g][r]), lds_u32(&sm.xt[g + 8][r]), lds_u32(&sm.xt[g][r + 8]),
+                                   lds_u32(&sm.xt[g + 8][r + 8])};
+            const uint32_t b[2] = {lds_u32(&sm.d1t[u0 + g][r]), lds_u32(&sm.d1t[u0 + g][r + 8])};
+            mma_bf16(c, x, b);
+        }
+        *reinterpret_cast<float2*>(&gW1[g * kNH + u0 + 2 * t]) = make_float2(c[0], c[1]);
+        *reinterpret_cast<float2*>(&gW1[(g + 8) * kNH + u0 + 2 * t]) = make_float2(c[2], c[3]);
+    }
+    // the row sums, added over the row groups in a fixed order
+    if (tid < kNH) {
+        float s3 = 0.f, sb2 = 0.f, sb1 = 0.f;
+        for (int w = 0; w < kTcWarps; ++w) {
+            s3 += sm.red[w][0][tid];
+            sb2 += sm.red[w][1][tid];
+            sb1 += sm.red[w][2][tid];
+        }
+        gW3[tid] = s3;
+        gb2[tid] = sb2;
+        gb1[tid] = sb1;
+    } else if (tid == kNH) {
+        float sg = 0.f, sl = 0.f;
+        for (int w = 0; w < kTcWarps; ++w) {
+            sg += sm.red_s[w][0];
+            sl += sm.red_s[w][1];
+        }
+        gW3[kNH] = sg;                // db3
+        ts.loss = sl;
+    }
+}
+
+__device__ __forceinline__ void cp_async(void* dst, const void* src, int bytes) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if (bytes == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+
+__global__ void __launch_bounds__(kTrainThreads) train_kernel(float* theta, float* am, float* av, const float* X,
+                                                        const float* yv, int count, int batch, int steps, int adam0,
+                                                        float lr, uint32_t k0, uint32_t k1, float* loss) {
+    extern __shared__ __align__(16) unsigned char tc_raw[];
+    TrainSmem& sm = *reinterpret_cast<TrainSmem*>(tc_raw);
+    cg::cluster_group cluster = cg::this_cluster();
+    const int ranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int g = lane >> 2, t = lane & 3, pair = warp & 3;
+    const int share = (kNParams + ranks - 1) / ranks;
+    const int i0 = rank * share, n_own = max(0, min(share, kNParams - i0));
+    float *own_t = sm.own, *own_m = own_t + share, *own_v = own_m + share;
+    for (int i = tid; i < kNParams; i += kTrainThreads) tc_store_param(sm.tc, i, theta[i]);
+    for (int i = tid; i < n_own; i += kTrainThreads) {
+        own_t[i] = theta[i0 + i];
+        own_m[i] = am[i0 + i];
+        own_v[i] = av[i0 + i];
+    }
+    const int my_row = rank * kTcRows + tid;   // of the mini-batch
+    auto request = [&](int step, int slot) {
+        if (tid < kTcRows && my_row < batch) {
+            const U4 u = philox(uint32_t(my_row), uint32_t(adam0 + 1 + step), 0u, 6u, k0, k1);
+            const int src = (int)(((unsigned long long)u.x * (unsigned)count) >> 32);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) cp_async(&sm.x[slot][tid][4 * q], X + size_t(src) * kNF + 4 * q, 16);
+            cp_async(&sm.y[slot][tid], yv + src, 4);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    request(0, 0);
+    const float scale = 1.0f / (float)batch;
+    for (int k = 0; k < steps; ++k) {
+        const int slot = k & 1;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();   // the rows of this step, from every thread
+        uint32_t ax[2][4];
+        float y[2][2];
+        bool act[2][2];
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int r = pair * 32 + 16 * mt + g + 8 * h;
+                act[mt][h] = rank * kTcRows + r < batch;
+                float2 lo = make_float2(0.f, 0.f), hi = make_float2(0.f, 0.f);
+                y[mt][h] = 0.f;
+                if (act[mt][h]) {
+                    lo = *reinterpret_cast<const float2*>(&sm.x[slot][r][2 * t]);
+                    hi = *reinterpret_cast<const float2*>(&sm.x[slot][r][2 * t + 8]);
+                    y[mt][h] = sm.y[slot][r];
+                }
+                tc_row(sm.tc, ax, mt, h, lo, hi, pair, g, t);   // (both halves write the same)
+            }
+        }
+        if (k + 1 < steps) request(k + 1, slot ^ 1);
+        train_gradient(sm, ax, act, y, scale, tid);
+        cluster.sync();   // every CTA's gradient
+        const float c1 = 1.f - powf(0.9f, (float)(adam0 + 1 + k)), c2 = 1.f - powf(0.999f, (float)(adam0 + 1 + k));
+        for (int i = tid; i < n_own; i += kTrainThreads) {
+            // the eight requests leave together (one after the other they were
+            // half of a step's time); absent CTAs repeat this one's
+            float part[kMaxTrainCtas];
+#pragma unroll
+            for (int b = 0; b < kMaxTrainCtas; ++b)
+                part[b] = cluster.map_shared_rank(sm.grad, b < ranks ? b : rank)[i0 + i];
+            float gr = 0.f;
+#pragma unroll
+            for (int b = 0; b < kMaxTrainCtas; ++b)
+                if (b < ranks) gr += part[b];
+            adam_update(gr, c1, c2, lr, own_m[i], own_v[i], own_t[i]);
+            for (int b = 0; b < ranks; ++b) tc_store_param(*cluster.map_shared_rank(&sm.tc, b), i0 + i, own_t[i]);
+        }
+        if (rank == 0 && tid == 0) {
+            float tot = 0.f;
+            for (int b = 0; b < ranks; ++b) tot += *cluster.map_shared_rank(&sm.loss, b);
+            loss[k] = tot;
+        }
+        cluster.sync();   // every CTA's operands; the gradients are read
+    }
+    for (int i = tid; i < n_own; i += kTrainThreads) {
+        theta[i0 + i] = own_t[i];
+        am[i0 + i] = own_m[i];
+        av[i0 + i] = own_v[i];
+    }
+}
+
+// Sum the per-CTA gradients in a fixed order; optionally take an Adam step.
 __global__ void reduce_adam_kernel(const float* partial, const float* partial_loss, int nblk, float* grad,
                                    float* loss, float* theta, float* m, float* v, int adam_t, float lr) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -645,14 +1136,7 @@ __global__ void reduce_adam_kernel(const float* partial, const float* partial_lo
     for (int b = 0; b < nblk; ++b) g += partial[size_t(b) * kNParams + i];
     if (grad) grad[i] = g;
     if (adam_t > 0) {
-        const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-        const float mi = b1 * m[i] + (1.f - b1) * g;
-        const float vi = b2 * v[i] + (1.f - b2) * g * g;
-        m[i] = mi;
-        v[i] = vi;
-        const float mh = mi / (1.f - powf(b1, (float)adam_t));
-        const float vh = vi / (1.f - powf(b2, (float)adam_t));
-        theta[i] -= lr * mh / (sqrtf(vh) + eps);
+        adam_update(g, 1.f - powf(0.9f, (float)adam_t), 1.f - powf(0.999f, (float)adam_t), lr, m[i], v[i], theta[i]);
     }
 }
 
@@ -735,6 +1219,38 @@ cudaError_t surrogate_step(const float* theta_in, const float* X, const float* y
     reduce_adam_kernel<<<(kNParams + 255) / 256, 256, 0, s>>>(partial, partial_loss, nblk, grad, loss, theta, m, v,
                                                               adam_t, lr);
     return cudaGetLastError();
+}
+
+namespace {
+
+size_t train_smem(int ranks) {
+    return sizeof(TrainSmem) + 3 * size_t((kNParams + ranks - 1) / ranks) * sizeof(float);
+}
+
+}  // namespace
+
+bool surrogate_train_fits(int batch) { return batch <= kMaxTrainCtas * kTcRows; }
+
+cudaError_t surrogate_train_steps(float* theta, float* m, float* v, const float* X, const float* y, int count,
+                                  int batch, int steps, int adam_t, float lr, uint32_t k0, uint32_t k1, float* loss,
+                                  cudaStream_t s) {
+    const int ranks = (batch + kTcRows - 1) / kTcRows;
+    if (ranks < 1 || ranks > kMaxTrainCtas) return cudaErrorInvalidValue;
+    const size_t smem = train_smem(ranks);
+    cudaError_t err = cudaFuncSetAttribute(train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ranks);
+    cfg.blockDim = dim3(kTrainThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = ranks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, train_kernel, theta, m, v, X, y, count, batch, steps, adam_t, lr, k0, k1, loss);
 }
 
 cudaError_t surrogate_init(float* theta, float scale, uint32_t k0, uint32_t k1, cudaStream_t s) {
