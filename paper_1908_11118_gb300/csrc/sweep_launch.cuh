@@ -8,10 +8,12 @@ namespace {
 
 // Registers per thread are bounded so that every walker that fits in shared
 // memory is resident: a direct walker takes 3-5 KB, so up to 28 one-warp CTAs
-// share an SM; four warps per walker run at about one walker per SM.
+// share an SM (a launch of 4096 walkers, 27 per SM: 24 resident 444 us on
+// fcc(100) and 571 us of clusters, 28 resident 366 and 507 us, the spills of 72
+// registers included); four warps per walker run at a few walkers per SM.
 template <int K, bool DA, bool CL, bool DIRECT>
 constexpr int min_ctas() {
-    return DIRECT && K == 1 ? 24 : (K == 4 ? 3 : 1);
+    return DIRECT && K == 1 ? 28 : (K == 4 ? 3 : 1);
 }
 
 template <int K, bool TRACE, bool DA, bool CL, bool DIRECT>

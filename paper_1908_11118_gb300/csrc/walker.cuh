@@ -37,11 +37,11 @@
 // fixed latency, 1.0 for shared memory or a shuffle, 0.4 for a branch, 0.3 for
 // the instruction fetch); it took 645 at 5.3 with a committing thread fed
 // through shared memory and the draws made one move at a time.  Steps of ten
-// sweeps, before / after: 16 fcc(100) replicas 406 / 248 us with the walkers read
+// sweeps, before / after: 16 fcc(100) replicas 406 / 243 us with the walkers read
 // back, a hundred REGC steps of 160 A18 replicas 2.2 / 1.1 ms, 4096 clusters
-// 950 / 620 us, the 1024-replica grid 400 / 377 us.  With delayed acceptance the
+// 950 / 555 us, the 1024-replica grid 400 / 375 us.  With delayed acceptance the
 // code of the features stands once instead of six times and the kernel is no
-// longer bound by the instruction fetch: 1930 / 915 us.
+// longer bound by the instruction fetch: 1930 / 864 us.
 #pragma once
 
 #include "cells.cuh"
@@ -58,7 +58,7 @@ constexpr int kRing = 64;                         // drawn moves kept ahead
 
 // One drawn move: two 16-byte words of the ring.
 struct Draw {
-    float x, y, z;    // displacement, or the insertion point
+    float x, y, z;    // displacement (0 for a removal), or the insertion point
     unsigned kind;    // bits 0-1 the type (0 displacement, 1 insertion, 2 removal), bit 2 the second species
     unsigned b0;      // Philox word picking the particle
     unsigned b1;      // Philox word of the acceptance
@@ -333,13 +333,14 @@ __device__ __forceinline__ void draw_moves(const SweepParams& P, const Hot& H, u
         if (d.x >= H.g.Lx) d.x = __fsub_rn(d.x, H.g.Lx);
         if (d.y >= H.g.Ly) d.y = __fsub_rn(d.y, H.g.Ly);
         if (H.g.periodic_z && d.z >= H.g.Lz) d.z = __fsub_rn(d.z, H.g.Lz);
+        if (type == 2u) d.x = d.y = d.z = 0.f;
     }
     // the species of a grand-canonical move: the second (the gas after a
     // cluster), or with two grand-canonical species the one bit 30 of B2 picks
     const unsigned gy = (CL && P.gc2) ? (B.z >> 30) & 1u : 1u;
     d.kind = type | (gy << 2);
     d.lu = __logf(((float)B.y + 0.5f) * 2.3283064365386963e-10f);
-    uint4* out = ring + 2 * (m % kRing);
+    uint4* out = ring + 2 * ((unsigned)m % kRing);
     out[0] = make_uint4(__float_as_uint(d.x), __float_as_uint(d.y), __float_as_uint(d.z), d.kind);
     out[1] = make_uint4(B.x, B.y, __float_as_uint(d.lu), B.w);
 }
@@ -358,14 +359,28 @@ __device__ __forceinline__ void draw_moves(const SweepParams& P, const Hot& H, u
 // Both compute a displacement rounded once from the same exact operands, so an
 // in-range pair term is the same bit for bit.
 
-// This lane's place in the 3 x 3 x 3 stencil.
+// This lane's place in the 3 x 3 x 3 stencil, and what wrapping its coordinate
+// around the grid adds to it: to the cell, and as the entry's shift.
 struct LaneCell {
     int x, y, z;
     bool in;
+    int wx, wy, wz;
+    float sx, sy, sz;
 };
 
-__device__ __forceinline__ LaneCell lane_cell(int lane) {
-    return LaneCell{lane % 3 - 1, (lane / 3) % 3 - 1, lane / 9 - 1, lane < 27};
+__device__ __forceinline__ LaneCell lane_cell(const Hot& H, int lane) {
+    LaneCell l;
+    l.x = lane % 3 - 1;
+    l.y = (lane / 3) % 3 - 1;
+    l.z = lane / 9 - 1;
+    l.in = lane < 27;
+    l.wx = l.x < 0 ? H.cg.ncx : -H.cg.ncx;
+    l.wy = l.y < 0 ? H.cg.ncy : -H.cg.ncy;
+    l.wz = l.z < 0 ? H.cg.ncz : -H.cg.ncz;
+    l.sx = l.x < 0 ? -H.g.Lx : H.g.Lx;
+    l.sy = l.y < 0 ? -H.g.Ly : H.g.Ly;
+    l.sz = l.z < 0 ? -H.g.Lz : H.g.Lz;
+    return l;
 }
 
 // The stencil of cell c as a list of its non-empty cells in st: {slot base,
@@ -377,32 +392,36 @@ __device__ __forceinline__ LaneCell lane_cell(int lane) {
 __device__ __forceinline__ int stencil_list(const Hot& H, const uint16_t* cnts, Cell3 c, LaneCell lc, int lane,
                                             float4* st, int& cnt, int& excl) {
     int ix = c.x + lc.x, iy = c.y + lc.y, iz = c.z + lc.z;
-    float sx = 0.f, sy = 0.f, sz = 0.f;
+    const bool wx = (unsigned)ix >= (unsigned)H.cg.ncx, wy = (unsigned)iy >= (unsigned)H.cg.ncy;
+    const bool wz = (unsigned)iz >= (unsigned)H.cg.ncz;
+    ix = wx ? ix + lc.wx : ix;
+    iy = wy ? iy + lc.wy : iy;
+    const float sx = wx ? lc.sx : 0.f, sy = wy ? lc.sy : 0.f;
+    float sz = 0.f;
     bool in = lc.in;
-    if (ix < 0) { ix += H.cg.ncx; sx = -H.g.Lx; }
-    else if (ix >= H.cg.ncx) { ix -= H.cg.ncx; sx = H.g.Lx; }
-    if (iy < 0) { iy += H.cg.ncy; sy = -H.g.Ly; }
-    else if (iy >= H.cg.ncy) { iy -= H.cg.ncy; sy = H.g.Ly; }
     if (H.g.periodic_z) {
-        if (iz < 0) { iz += H.cg.ncz; sz = -H.g.Lz; }
-        else if (iz >= H.cg.ncz) { iz -= H.cg.ncz; sz = H.g.Lz; }
+        iz = wz ? iz + lc.wz : iz;
+        sz = wz ? lc.sz : 0.f;
     } else {
-        in = in && iz >= 0 && iz < H.cg.ncz;
+        in = in && !wz;
     }
     const int cell = (iz * H.cg.ncy + iy) * H.cg.ncx + ix;
     cnt = in ? (int)cnts[cell] : 0;
+    const int total = (int)__reduce_add_sync(FULL, (unsigned)cnt);
     int incl = cnt;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(FULL, incl, o);
-        if (lane >= o) incl += t;
-    }
+    for (int o = 1; o < 32; o <<= 1)   // inclusive scan; the shuffle's predicate says which lanes have a source
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t.reg .b32 t;\n\t"
+            "shfl.sync.up.b32 t|p, %0, %1, 0, 0xffffffff;\n\t"
+            "@p add.s32 %0, %0, t;\n\t}"
+            : "+r"(incl)
+            : "r"(o));
     excl = incl - cnt;
     const unsigned nonempty = __ballot_sync(FULL, cnt > 0);
     if (cnt > 0)
         st[__popc(nonempty & lanemask_lt(lane))] =
             make_float4(__int_as_float(cell * H.cg.cap - excl), sx, sy, sz);
-    const int total = __shfl_sync(FULL, incl, 31);
     __syncwarp();
     return total;
 }
@@ -617,50 +636,42 @@ __device__ __forceinline__ Trial evaluate_move(const SweepParams& P, const Hot& 
     // displacement; insertion and removal act on the gas after it) or two
     // grand-canonical species B and C (split = N_B, gc2).
     const int split = CL ? split_in : 0;
-    const uint4 d0 = S.ring[2 * (m % kRing)], d1 = S.ring[2 * (m % kRing) + 1];
+    const uint4 d0 = S.ring[2 * ((unsigned)m % kRing)], d1 = S.ring[2 * ((unsigned)m % kRing) + 1];
     Trial r;
     const int type = (int)(d0.w & 3u);
     const int gy = CL ? (int)((d0.w >> 2) & 1u) : 1;
     const int gcnt = gy ? N - split : split;          // the species' count before the move
     const bool use2 = CL && P.gc2 && gy == 1;         // species C's constants
     const float cins_f = use2 ? sf.c_ins2 : sf.c_ins, cdel_f = use2 ? sf.c_del2 : sf.c_del;
-    const float dx = __uint_as_float(d0.x), dy = __uint_as_float(d0.y), dz = __uint_as_float(d0.z);
     r.b1 = d1.y;
     r.lu = __uint_as_float(d1.z);
     r.b3 = d1.w;
+    // One path for the three kinds, without branches: the new position is the
+    // particle's (an insertion: 0) plus the drawn numbers; what a kind does not
+    // need is read from particle 0 and dropped.
+    const bool disp = type == 0, ins = type == 1;
     // the particle: any of N for a displacement, of the species for a removal
-    const int pick_n = type == 0 ? N : gcnt, pick_0 = (type == 2 && gy) ? split : 0;
-    int idx = -1, status = 0;
-    float4 old = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (type != 1) {
-        if (pick_n == 0) {
-            status = 1;
-        } else {
-            idx = pick_0 + (int)(((unsigned long long)d1.x * (unsigned)pick_n) >> 32);
-            old = S.pos[idx];
-        }
-    } else if (N == H.nmax) {
-        status = 1;
-    }
-    float qx = old.x, qy = old.y, qz = old.z;
-    if (type == 0 && status == 0) {
-        qx = __fadd_rn(old.x, dx);
-        qy = __fadd_rn(old.y, dy);
-        qz = __fadd_rn(old.z, dz);
-        if (qx < 0.f) qx = __fadd_rn(qx, H.g.Lx);
-        if (qx >= H.g.Lx) qx = __fsub_rn(qx, H.g.Lx);
-        if (qy < 0.f) qy = __fadd_rn(qy, H.g.Ly);
-        if (qy >= H.g.Ly) qy = __fsub_rn(qy, H.g.Ly);
-        if (H.g.periodic_z) {
-            if (qz < 0.f) qz = __fadd_rn(qz, H.g.Lz);
-            if (qz >= H.g.Lz) qz = __fsub_rn(qz, H.g.Lz);
-        } else if (qz < H.g.z_lo || qz > H.g.z_hi) {
-            status = 2;
-        }
-    } else if (type == 1 && status == 0) {
-        qx = dx;
-        qy = dy;
-        qz = dz;
+    const int pick_n = disp ? N : gcnt, pick_0 = (type == 2 && gy) ? split : 0;
+    int status = (ins ? N == H.nmax : pick_n == 0) ? 1 : 0;
+    const int idx = (ins || status) ? -1 : pick_0 + (int)__umulhi(d1.x, (unsigned)pick_n);
+    float4 old = S.pos[max(idx, 0)];
+    if (ins) old = make_float4(0.f, 0.f, 0.f, 0.f);
+    // ln of the count factor with its constant, ready for the decision
+    const float lg = __logf((float)(gcnt + (ins ? 1 : 0)));
+    const float c_gc = disp ? 0.f : (ins ? cins_f - lg : cdel_f + lg);
+    float qx = __fadd_rn(old.x, __uint_as_float(d0.x));
+    float qy = __fadd_rn(old.y, __uint_as_float(d0.y));
+    float qz = __fadd_rn(old.z, __uint_as_float(d0.z));
+    // (an insertion's point and a removed particle's are inside already)
+    qx = qx < 0.f ? __fadd_rn(qx, H.g.Lx) : qx;
+    qx = qx >= H.g.Lx ? __fsub_rn(qx, H.g.Lx) : qx;
+    qy = qy < 0.f ? __fadd_rn(qy, H.g.Ly) : qy;
+    qy = qy >= H.g.Ly ? __fsub_rn(qy, H.g.Ly) : qy;
+    if (H.g.periodic_z) {
+        qz = qz < 0.f ? __fadd_rn(qz, H.g.Lz) : qz;
+        qz = qz >= H.g.Lz ? __fsub_rn(qz, H.g.Lz) : qz;
+    } else if (disp && status == 0 && (qz < H.g.z_lo || qz > H.g.z_hi)) {
+        status = 2;
     }
     const bool two_q = type == 0;
     // pair tables of the moving species
@@ -695,7 +706,7 @@ __device__ __forceinline__ Trial evaluate_move(const SweepParams& P, const Hot& 
         const float e0 = net_mma(*nf, a, &e1);
         dEs = type == 1 ? e0 : (type == 2 ? -e0 : e0 - e1);
         // ln u1 < ln alpha with dE~ in place of dE (u1 from B3)
-        const float la1 = count_term(type, gcnt, cins_f, cdel_f) - sf.beta * dEs;
+        const float la1 = c_gc - sf.beta * dEs;
         const float lu1 = __logf(((float)r.b3 + 0.5f) * 2.3283064365386963e-10f);
         if (la1 >= 0.f || lu1 < la1 - 1e-3f) stage1 = 1;
         else if (lu1 > la1 + 1e-3f) stage1 = 0;
@@ -715,10 +726,16 @@ __device__ __forceinline__ Trial evaluate_move(const SweepParams& P, const Hot& 
         // the surface columns are requested first: they come from L2 while the
         // mobile partners are evaluated
         const bool s0 = near_surf(H, qz), s1 = two_q && near_surf(H, old.z);
-        const int col0 = s0 ? surf_slot(H, qx, qy) : 0, col1 = s1 ? surf_slot(H, old.x, old.y) : 0;
-        float4 a0 = make_float4(0.f, 0.f, 1e30f, __uint_as_float(32u)), a1 = a0;
-        if (s0) a0 = __ldg(&H.st.atoms[col0 + lane]);
-        if (s1) a1 = __ldg(&H.st.atoms[col1 + lane]);
+        int col0 = 0, col1 = 0;
+        float4 a0, a1;
+        if (s0) {
+            col0 = surf_slot(H, qx, qy);
+            a0 = __ldg(&H.st.atoms[col0 + lane]);
+        }
+        if (s1) {
+            col1 = surf_slot(H, old.x, old.y);
+            a1 = __ldg(&H.st.atoms[col1 + lane]);
+        }
         if (DIRECT) {
             if (H.cg.cap < H.nmax) c_new = cell_lin(H, cell3_hot(H, qx, qy, qz));
             if (two_q)
@@ -796,7 +813,7 @@ __device__ __forceinline__ Trial evaluate_move(const SweepParams& P, const Hot& 
     if (status == 0 && !ovl) {
         const float de_f = fix_to_f32(big, hi, lo);
         if (!DA) {
-            r.dec = pretest(count_term(type, gcnt, cins_f, cdel_f), sf.beta, de_f, r.lu);
+            r.dec = pretest(c_gc, sf.beta, de_f, r.lu);
         } else if (stage1) {
             // stage 2: ln u2 < -beta (dE - dE~) (u2 from B1)
             const float la2 = -sf.beta * (de_f - dEs);
@@ -1122,7 +1139,7 @@ __device__ __forceinline__ void walker_sweep(const SweepParams& P, int w, char* 
     }
     group_sync<K>(bar);
 
-    const LaneCell lc = lane_cell(lane);
+    const LaneCell lc = lane_cell(H, lane);
     int n_cand = 0;
     NetFrag nf;                       // the surrogate's weights in this lane's fragments
     if (DA) load_net(P.net, lane, nf);
