@@ -36,7 +36,7 @@ struct Bucket {
     int wpc = 1, grid = 1;          // walkers per CTA, CTAs
     double ms = -1.0;               // last measured kernel time
     struct Shape {
-        int k, wpc, region;
+        int k, wpc, region, occ;    // occ: resident CTAs per SM
     };
     std::vector<Shape> cand;        // feasible (warps per walker, walkers per CTA) choices
 };
@@ -284,33 +284,67 @@ regc_status regc_batch_create(regc_handle* const* handles, int count, int sweeps
     if (e == cudaSuccess) e = batch_prepare((int)kMaxSmem);
     // feasible shapes (warps per walker 1, 2, 4 -- more than one only for
     // plain one-species classes -- times walkers per CTA, CTAs of at most 16
-    // warps), and the default: one warp per walker, the most resident walkers
-    // per SM
+    // warps)
     for (auto& q : b->buckets) {
-        int best = 0;
-        const size_t stat = batch_static_smem(q.c.da);
+        for (int m : q.members)
+            if (!batch_admits(handles[m]->P) && e == cudaSuccess) e = cudaErrorInvalidValue;
         for (int k = 1; k <= 4 && e == cudaSuccess; k *= 2) {
             if (k > 1 && (q.c.da || q.c.cl)) break;
             size_t region = 0;
             for (int m : q.members) region = std::max(region, sweep_smem(handles[m]->P, k));
-            region = (region + 15) / 16 * 16;
+            region = (region + batch_head() + 15) / 16 * 16;
             for (int wpc = 1; k * wpc <= batch_max_warps(q.c.da) && e == cudaSuccess; wpc *= 2) {
-                if ((size_t)wpc * region + stat > kMaxSmem) break;
+                if ((size_t)wpc * region > kMaxSmem) break;
                 const int occ = batch_occupancy(wpc, k, (int)region, q.c);
                 if (occ < 1) break;
-                q.cand.push_back({k, wpc, (int)region});
-                if (k == 1 && wpc * occ > best) {
-                    best = wpc * occ;
-                    q.k = 1;
-                    q.wpc = wpc;
-                    q.region = (int)region;
-                }
+                q.cand.push_back({k, wpc, (int)region, occ});
             }
         }
         if (q.cand.empty()) e = cudaErrorInvalidValue;   // one walker does not fit
-        const int occ = batch_occupancy(q.wpc, q.k, q.region, q.c);
-        const int need = (int)((q.items.size() + q.wpc - 1) / q.wpc);
-        q.grid = std::max(1, std::min(need, b->sms * std::max(occ, 1)));
+    }
+    // The default shapes.  A class's walkers are spread over the SMs: the fewest
+    // walkers per CTA with which all of them are resident, else the most
+    // resident ones.  (The most resident per SM, as it was, put a small class of
+    // walkers into a few CTAs on a few of the SMs.)  The classes run side by
+    // side and the slowest chains, those of the largest Nmax, end the step, so
+    // spare issue slots go to the largest classes: four warps per walker while
+    // the batch then has at most 14 warps per SM (3.5 walkers of four, where a
+    // single system's choice lies), else two.  A step of ten sweeps of 16, 64,
+    // 160, 256 uneven systems (Nmax 64 .. 2048) with the default shapes, one warp
+    // per walker in every class before / so: 0.61 / 0.30, 1.10 / 0.98, 2.46 /
+    // 1.60, 4.20 / 2.45 ms (autotuned: 0.30, 0.79, 1.53, 2.41).
+    if (e == cudaSuccess) {
+        auto shape = [&](const Bucket& q, int k) {
+            const Bucket::Shape* best = nullptr;
+            for (const auto& c : q.cand) {
+                if (c.k != k) continue;
+                const long long room = (long long)c.wpc * c.occ * b->sms;
+                if (!best || (long long)best->wpc * best->occ * b->sms < (long long)q.items.size()) {
+                    if (!best || room > (long long)best->wpc * best->occ * b->sms) best = &c;
+                }
+            }
+            return best;
+        };
+        auto warps_per_sm = [&](const Bucket& q, const Bucket::Shape& c) {
+            return c.k * std::min((double)q.items.size() / b->sms, (double)c.wpc * c.occ);
+        };
+        double rest = 0.0;   // warps per SM of the classes not yet settled, at one warp per walker
+        for (auto& q : b->buckets) rest += warps_per_sm(q, *shape(q, 1));
+        double used = 0.0;
+        for (auto& q : b->buckets) {
+            rest -= warps_per_sm(q, *shape(q, 1));
+            const Bucket::Shape* pick = shape(q, 1);
+            for (int k = 2; k <= 4; k *= 2) {
+                const Bucket::Shape* c = shape(q, k);
+                if (c && used + warps_per_sm(q, *c) + rest <= 14.0) pick = c;
+            }
+            used += warps_per_sm(q, *pick);
+            q.k = pick->k;
+            q.wpc = pick->wpc;
+            q.region = pick->region;
+            const int need = (int)((q.items.size() + q.wpc - 1) / q.wpc);
+            q.grid = std::max(1, std::min(need, b->sms * pick->occ));
+        }
     }
     const int nb = (int)b->buckets.size();
     if (e == cudaSuccess) e = cudaMalloc(&b->d_sys, count * sizeof(SweepParams));
@@ -390,12 +424,11 @@ regc_status regc_batch_autotune(regc_batch* b, int rounds) {
         for (size_t c = 0; c < n_cand; ++c) {
             for (auto& q : b->buckets) {
                 const Bucket::Shape sh = q.cand[std::min(c, q.cand.size() - 1)];
-                const int occ = batch_occupancy(sh.wpc, sh.k, sh.region, q.c);
                 const int need = (int)((q.items.size() + sh.wpc - 1) / sh.wpc);
                 q.k = sh.k;
                 q.wpc = sh.wpc;
                 q.region = sh.region;
-                q.grid = std::max(1, std::min(need, b->sms * std::max(occ, 1)));
+                q.grid = std::max(1, std::min(need, b->sms * sh.occ));
             }
             st = fail(b, record_step(b, &ms));
             if (st != REGC_OK) return st;
@@ -403,7 +436,7 @@ regc_status regc_batch_autotune(regc_batch* b, int rounds) {
             for (int k = 0; k < nb; ++k)
                 if (ms[k] < best[k]) {
                     best[k] = ms[k];
-                    best_shape[k] = {b->buckets[k].k, b->buckets[k].wpc, b->buckets[k].region};
+                    best_shape[k] = {b->buckets[k].k, b->buckets[k].wpc, b->buckets[k].region, 0};
                     best_grid[k] = b->buckets[k].grid;
                 }
         }

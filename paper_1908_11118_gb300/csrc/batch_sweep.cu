@@ -8,8 +8,8 @@ namespace {
 // Persistent sweep of a batch of walkers from several systems.  Every group
 // of K warps of the CTA is one walker at a time: its first thread takes the
 // next (system, walker) item from the queue, the group copies that system's
-// parameters into its slot of shared memory and runs the walker's sweeps in
-// its own shared-memory region of `region` bytes (K > 1: the speculative
+// parameters to the head of its shared-memory region of `region` bytes and runs
+// the walker's sweeps in the rest of it (K > 1: the speculative
 // walker, synchronised by the group's named barrier 1 + group); items are
 // listed largest first, so the queue balances the uneven costs.  DA: the
 // systems of the launch sample with delayed acceptance (their networks'
@@ -18,43 +18,48 @@ namespace {
 // DIRECT: its walkers enumerate all particles instead of a cell list.
 constexpr int kBatchMaxWarps = 16;
 constexpr int kBatchMaxWarpsDA = 4;
+constexpr int kBatchHead = (int)((sizeof(SweepParams) + sizeof(int) + 15) / 16 * 16);   // parameters and item
 
 template <bool DA, bool CL, bool DIRECT, int K>
 __global__ void __launch_bounds__(32 * (DA ? kBatchMaxWarpsDA : kBatchMaxWarps))
     batch_sweep_kernel(const SweepParams* __restrict__ sys, const int2* __restrict__ items, int n_items,
                        int* counter, int region) {
-    constexpr int kGroups = (DA ? kBatchMaxWarpsDA : kBatchMaxWarps) / K;
     extern __shared__ __align__(16) char smem[];
-    __shared__ SweepParams Psh[kGroups];
-    __shared__ int item_sh[kGroups];
     const int tid = threadIdx.x % (32 * K), grp = threadIdx.x / (32 * K);
     const int bar = K == 1 ? 0 : 1 + grp;
     char* mine = smem + (size_t)grp * region;
+    SweepParams& Psh = *reinterpret_cast<SweepParams*>(mine);
+    int& item_sh = *reinterpret_cast<int*>(mine + sizeof(SweepParams));
     for (;;) {
         int item = 0;
         if (K == 1) {
             if (tid == 0) item = atomicAdd(counter, 1);
             item = __shfl_sync(FULL, item, 0);
         } else {
-            if (tid == 0) item_sh[grp] = atomicAdd(counter, 1);
+            if (tid == 0) item_sh = atomicAdd(counter, 1);
             group_sync<K>(bar);
-            item = item_sh[grp];
+            item = item_sh;
         }
         if (item >= n_items) break;
         const int2 mw = items[item];
         const int* src = reinterpret_cast<const int*>(sys + mw.x);
-        int* dst = reinterpret_cast<int*>(&Psh[grp]);
+        int* dst = reinterpret_cast<int*>(mine);
         for (int k = tid; k < (int)(sizeof(SweepParams) / sizeof(int)); k += 32 * K) dst[k] = src[k];
         group_sync<K>(bar);
-        walker_sweep<K, false, DA, CL, DIRECT>(Psh[grp], mw.y, mine, tid, bar);
+        walker_sweep<K, false, DA, CL, DIRECT>(Psh, mw.y, mine + kBatchHead, tid, bar);
         group_sync<K>(bar);   // the slot and the item are rewritten for the next walker
     }
 }
 
 }  // namespace
 
-size_t batch_static_smem(bool da) {
-    return (sizeof(SweepParams) + sizeof(int)) * (da ? kBatchMaxWarpsDA : kBatchMaxWarps);
+size_t batch_head() { return kBatchHead; }
+
+// A system joins a batch where its walker was admitted beside the parameter
+// blocks (756 bytes each) of a CTA's most walkers; the regions in use need less.
+bool batch_admits(const SweepParams& P) {
+    const int groups = P.delayed ? kBatchMaxWarpsDA : kBatchMaxWarps;
+    return align16(sweep_smem_admitted(P.nmax, P.cg.ncell, P.cg.cap, 1)) + (size_t)756 * groups <= 232448;
 }
 
 int batch_max_warps(bool da) { return da ? kBatchMaxWarpsDA : kBatchMaxWarps; }
@@ -86,7 +91,7 @@ struct Prepare {
         if (err == cudaSuccess)
             err = cudaFuncSetAttribute(batch_sweep_kernel<DA, CL, DIRECT, K>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       max_smem - (int)batch_static_smem(DA));
+                                       max_smem);
     }
 };
 

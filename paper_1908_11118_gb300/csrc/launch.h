@@ -60,9 +60,12 @@ cudaError_t pack_walkers(const float* xyz, const int* n, int S, int nmax, const 
 cudaError_t unpack_walkers(const float4* pos, long long count, int nmax, const int* n, float* xyz, cudaStream_t s);
 
 // ---------------------------------------------------------------- batch
-// Static shared memory of the batch sweep kernel and its warp limit per CTA
-// (da: the delayed-acceptance instantiation).
-size_t batch_static_smem(bool da);
+// Bytes at the head of a batch walker's region of shared memory (before
+// sweep_smem's), whether a system's walkers are admitted to a batch, and the
+// batch sweep kernel's warp limit per CTA (da: the delayed-acceptance
+// instantiation).
+size_t batch_head();
+bool batch_admits(const SweepParams& P);
 int batch_max_warps(bool da);
 
 // What the systems of one batch launch have in common: da, sampling with
