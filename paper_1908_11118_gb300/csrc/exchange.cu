@@ -97,7 +97,18 @@ __global__ void __launch_bounds__(256) batch_exchange_kernel(const ExchangeParam
     }
 }
 
+__global__ void batch_errors_kernel(const SweepParams* sys, int n_systems, int* out) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m < n_systems) out[m] = *sys[m].error;
+}
+
 }  // namespace
+
+cudaError_t batch_errors(const SweepParams* sys, int n_systems, int* out, cudaStream_t s) {
+    if (n_systems <= 0) return cudaSuccess;
+    batch_errors_kernel<<<(n_systems + 127) / 128, 128, 0, s>>>(sys, n_systems, out);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_batch_exchange(const ExchangeParams* xs, uint32_t* e_ctr, SweepParams* sys, int n_systems,
                                   int n_sweeps, cudaStream_t s) {

@@ -67,7 +67,7 @@ struct regc_handle {
     int* d_error = nullptr;
     long long* d_fix = nullptr;               // scratch [S] for energy recomputes
     float* d_xyz = nullptr;                   // staging [S][nmax][3] for walker I/O
-    void* h_stage = nullptr;                  // pinned host staging: error word, [S] energies or labels
+    void* h_stage = nullptr;                  // pinned host staging: error word, walkers or counters read back, labels
     // learned surrogate (delayed acceptance)
     bool has_sur = false;
     float* d_theta = nullptr;                 // [5313] binary32 master parameters
@@ -101,6 +101,9 @@ struct regc_handle {
 // Synchronise the handle's stream and fold its device error word into the
 // sticky status.
 regc_status handle_sync_check(regc_handle* h);
+
+// Fold a device error word into the handle's sticky status.
+regc_status handle_fold_error(regc_handle* h, int err);
 
 // Record a CUDA error as the handle's sticky status; returns the status.
 regc_status handle_cuda_fail(regc_handle* h, cudaError_t e);

@@ -55,9 +55,25 @@ cudaError_t launch_energy(const SweepParams& P, long long* out, int check_overla
 cudaError_t pack_walkers(const float* xyz, const int* n, int S, int nmax, const Geometry& g, float4* pos, int* error,
                          cudaStream_t s);
 
-// pos [count] -> xyz [count][3] (count = S nmax); with n [S], only the first
-// n[w] entries of each walker are written.
-cudaError_t unpack_walkers(const float4* pos, long long count, int nmax, const int* n, float* xyz, cudaStream_t s);
+// What a read-back returns beside positions: arrays of 32-bit words (words[q]
+// of them, 0: none), energies (null: none) and the error word, to host memory
+// the device can write (page-locked).
+struct ReadBack {
+    static constexpr int kSegs = 3;
+    const unsigned* src[kSegs];
+    unsigned* dst[kSegs];
+    long long words[kSegs];
+    const long long* efix;   // [S] in units of 2^-30
+    double* energy;          // [S]
+    int S;
+    const int* error;
+    int* error_out;
+};
+
+// One launch: r, and (xyz given) pos [count] -> xyz [count][3] (count = S nmax);
+// with n [S], only the first n[w] entries of each walker are written.
+cudaError_t read_back(const float4* pos, long long count, int nmax, const int* n, float* xyz, const ReadBack& r,
+                      cudaStream_t s);
 
 // ---------------------------------------------------------------- batch
 // Bytes at the head of a batch walker's region of shared memory (before
@@ -90,6 +106,9 @@ cudaError_t batch_prepare(int max_smem);
 
 // Resident CTAs per SM of the batch sweep kernel for this shape (0 if none fit).
 int batch_occupancy(int walkers_per_cta, int warps_per_walker, int region, BatchClass c);
+
+// out[m] = system m's error word (out: page-locked host memory).
+cudaError_t batch_errors(const SweepParams* sys, int n_systems, int* out, cudaStream_t s);
 
 // One exchange attempt of every system's grid (attempt numbers e_ctr[]), then
 // e_ctr[m] += 1 and sys[m].t0 += n_sweeps on the device.

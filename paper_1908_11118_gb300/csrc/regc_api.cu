@@ -47,6 +47,14 @@ regc_status upload(regc_handle* h, T* dst, const T* src, size_t count) {
     return cuda_fail(h, cudaMemcpyAsync(dst, src, count * sizeof(T), cudaMemcpyHostToDevice, h->stream));
 }
 
+// Fold a device error word into the sticky status.
+regc_status fold_error(regc_handle* h, int err) {
+    if (err & ERR_TIMEOUT) h->sticky = REGC_ETIMEOUT;
+    else if (err & ERR_CAPACITY) h->sticky = REGC_ECAPACITY;
+    else if (err & ERR_NUMERIC) h->sticky = REGC_ENUMERIC;
+    return h->sticky;
+}
+
 // Synchronise and fold the device error word into the sticky status.
 regc_status sync_check(regc_handle* h) {
     if (h->sticky != REGC_OK) return h->sticky;
@@ -54,12 +62,12 @@ regc_status sync_check(regc_handle* h) {
     cudaError_t e = cudaMemcpyAsync(flag, h->d_error, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e);
-    const int err = *flag;
-    if (err & ERR_TIMEOUT) h->sticky = REGC_ETIMEOUT;
-    else if (err & ERR_CAPACITY) h->sticky = REGC_ECAPACITY;
-    else if (err & ERR_NUMERIC) h->sticky = REGC_ENUMERIC;
-    return h->sticky;
+    return fold_error(h, *flag);
 }
+
+// Bytes of the page-locked staging area: the error word, then what a read-back
+// of the walkers or of the counters takes.
+size_t stage_bytes(int S) { return 64 + (size_t)S * 8 * 16 + 64; }
 
 int cells_along(double len, double rc) {
     const int n = (int)floor(len / (rc * 1.00001));
@@ -87,6 +95,8 @@ float hard_core_r2(double eps, double sigma, double T) {
 }  // namespace
 
 regc_status handle_sync_check(regc_handle* h) { return sync_check(h); }
+
+regc_status handle_fold_error(regc_handle* h, int err) { return fold_error(h, err); }
 
 regc_status handle_cuda_fail(regc_handle* h, cudaError_t e) { return cuda_fail(h, e); }
 
@@ -519,7 +529,7 @@ regc_status init_grid(const regc_potential* pot, const regc_surface* surf, const
     TRY(dalloc(h, &h->d_error, 1));
     TRY(dalloc(h, &h->d_fix, S));
     TRY(dalloc(h, &h->d_xyz, (size_t)S * grid->nmax * 3));
-    if (cudaHostAlloc(&h->h_stage, 64 + (size_t)S * 8, cudaHostAllocDefault) != cudaSuccess) {
+    if (cudaHostAlloc(&h->h_stage, stage_bytes(S), cudaHostAllocDefault) != cudaSuccess) {
         h->h_stage = nullptr;
         regc_free(h);
         return REGC_ENOMEM;
@@ -949,6 +959,55 @@ void* device_view(const void* host) {
     return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
+// A read-back's destinations: the caller's page-locked buffers, or places in the
+// handle's staging area that finish() copies from.
+struct ReadBackTo {
+    regc_handle* h;
+    ReadBack r{};
+    struct Staged {
+        void* to;
+        const void* from;
+        size_t bytes;
+    } staged[ReadBack::kSegs + 1];
+    int n_seg = 0, n_staged = 0;
+    size_t used = 64;
+
+    explicit ReadBackTo(regc_handle* handle) : h(handle) {
+        r.S = h->S;
+        r.error = h->d_error;
+        r.error_out = static_cast<int*>(h->h_stage);
+    }
+    void* place(void* to, size_t bytes) {
+        if (reinterpret_cast<uintptr_t>(to) % 8 == 0)
+            if (void* d = device_view(to)) return d;
+        void* p = static_cast<char*>(h->h_stage) + used;
+        used += (bytes + 7) / 8 * 8;
+        staged[n_staged++] = Staged{to, p, bytes};
+        return p;
+    }
+    // n 32-bit words of device memory to `to` (null: nothing)
+    void words(void* to, const void* from, size_t n) {
+        if (!to) return;
+        r.src[n_seg] = static_cast<const unsigned*>(from);
+        r.dst[n_seg] = static_cast<unsigned*>(place(to, n * 4));
+        r.words[n_seg++] = (long long)n;
+    }
+    void energies(double* to) {
+        if (!to) return;
+        r.efix = h->P.efix;
+        r.energy = static_cast<double*>(place(to, (size_t)h->S * 8));
+    }
+    // once the launch is queued: wait for it, hand out what was staged
+    regc_status finish() {
+        const cudaError_t e = cudaStreamSynchronize(h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e);
+        const regc_status st = fold_error(h, *static_cast<int*>(h->h_stage));
+        if (st != REGC_OK) return st;
+        for (int i = 0; i < n_staged; ++i) memcpy(staged[i].to, staged[i].from, staged[i].bytes);
+        return REGC_OK;
+    }
+};
+
 }  // namespace
 
 regc_status regc_set_walkers(regc_handle* h, const float* pos, const int32_t* n, const int32_t* sow) {
@@ -1040,29 +1099,20 @@ regc_status regc_get_walkers2(regc_handle* h, float* pos, int32_t* n, int32_t* n
     if (h->sticky != REGC_OK) return h->sticky;
     if (nb && !h->P.gc2) return REGC_EINVAL;
     const int S = h->S, nmax = h->nmax;
-    long long* ef = reinterpret_cast<long long*>(static_cast<char*>(h->h_stage) + 64);   // pinned
-    cudaError_t e = cudaSuccess;
-    if (pos) {
-        // a page-locked caller buffer is written in place by the unpacking kernel
-        float* dst = static_cast<float*>(device_view(pos));
-        e = unpack_walkers(h->P.pos, (long long)S * nmax, nmax, dst ? h->P.n : nullptr, dst ? dst : h->d_xyz,
-                           h->stream);
-        if (e == cudaSuccess && !dst)
-            e = cudaMemcpyAsync(pos, h->d_xyz, (size_t)S * nmax * 3 * sizeof(float), cudaMemcpyDeviceToHost,
-                                h->stream);
-    }
-    if (n && e == cudaSuccess) e = cudaMemcpyAsync(n, h->P.n, S * sizeof(int), cudaMemcpyDeviceToHost, h->stream);
-    if (nb && e == cudaSuccess) e = cudaMemcpyAsync(nb, h->P.nb, S * sizeof(int), cudaMemcpyDeviceToHost, h->stream);
-    if (energy && e == cudaSuccess)
-        e = cudaMemcpyAsync(ef, h->P.efix, S * sizeof(long long), cudaMemcpyDeviceToHost, h->stream);
-    if (sow && e == cudaSuccess)
-        e = cudaMemcpyAsync(sow, h->X.state_of_walker, S * sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+    // page-locked caller buffers are written in place by the kernel; the others
+    // (positions: by a copy) through the staging area
+    float* dst = pos ? static_cast<float*>(device_view(pos)) : nullptr;
+    ReadBackTo to(h);
+    to.words(n, h->P.n, S);
+    to.words(nb, h->P.nb, S);
+    to.words(sow, h->X.state_of_walker, S);
+    to.energies(energy);
+    cudaError_t e = read_back(h->P.pos, (long long)S * nmax, nmax, dst ? h->P.n : nullptr,
+                              pos ? (dst ? dst : h->d_xyz) : nullptr, to.r, h->stream);
+    if (e == cudaSuccess && pos && !dst)
+        e = cudaMemcpyAsync(pos, h->d_xyz, (size_t)S * nmax * 3 * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e);
-    const regc_status st = sync_check(h);
-    if (st != REGC_OK) return st;
-    if (energy)
-        for (int w = 0; w < S; ++w) energy[w] = (double)ef[w] * kFixUnit;
-    return REGC_OK;
+    return to.finish();
 }
 
 regc_status regc_check_energy(regc_handle* h, double* max_drift) {
@@ -1093,15 +1143,13 @@ regc_status regc_warps_per_walker(const regc_handle* h, int* warps) {
 regc_status regc_counters(regc_handle* h, int64_t* moves, int64_t* exchanges, int64_t* pairs) {
     if (!h) return REGC_EINVAL;
     if (h->sticky != REGC_OK) return h->sticky;
-    cudaError_t e = cudaSuccess;
-    if (moves) e = cudaMemcpyAsync(moves, h->P.move_counts, (size_t)h->S * 6 * 8, cudaMemcpyDeviceToHost, h->stream);
-    if (exchanges && e == cudaSuccess)
-        e = cudaMemcpyAsync(exchanges, h->X.ex_counts, (size_t)h->S * 2 * h->n_dir * 8, cudaMemcpyDeviceToHost,
-                            h->stream);
-    if (pairs && e == cudaSuccess)
-        e = cudaMemcpyAsync(pairs, h->P.pair_counts, 6 * 8, cudaMemcpyDeviceToHost, h->stream);
+    ReadBackTo to(h);
+    to.words(moves, h->P.move_counts, (size_t)h->S * 12);
+    to.words(exchanges, h->X.ex_counts, (size_t)h->S * 4 * h->n_dir);
+    to.words(pairs, h->P.pair_counts, 12);
+    const cudaError_t e = read_back(nullptr, 0, 1, nullptr, nullptr, to.r, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e);
-    return sync_check(h);
+    return to.finish();
 }
 
 // ------------------------------------------------------------ checkpoint

@@ -25,14 +25,26 @@ __global__ void pack_walkers_kernel(const float* xyz, const int* n, int S, int n
     pos[k] = v;
 }
 
-__global__ void unpack_walkers_kernel(const float4* pos, long long count, int nmax, const int* n, float* xyz) {
+// One launch for everything a call reads back: positions (where xyz is given;
+// with n only the first n[w] entries of each walker), energies, arrays copied
+// word by word and the error word, written straight to page-locked host memory.
+// Four copies and the error word's, one after the other on the copy engine,
+// were most of the 50 us that reading sixteen walkers took.
+__global__ void __launch_bounds__(256) read_back_kernel(const float4* pos, long long count, int nmax, const int* n,
+                                                        float* xyz, const __grid_constant__ ReadBack r) {
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= count) return;
-    if (n && (int)(k % nmax) >= n[k / nmax]) return;   // beyond N: left as it was
-    const float4 v = pos[k];
-    xyz[3 * k] = v.x;
-    xyz[3 * k + 1] = v.y;
-    xyz[3 * k + 2] = v.z;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    if (xyz && k < count && !(n && (int)(k % nmax) >= n[k / nmax])) {
+        const float4 v = pos[k];
+        xyz[3 * k] = v.x;
+        xyz[3 * k + 1] = v.y;
+        xyz[3 * k + 2] = v.z;
+    }
+    for (int q = 0; q < ReadBack::kSegs; ++q)
+        for (long long i = k; i < r.words[q]; i += stride) r.dst[q][i] = r.src[q][i];
+    if (r.energy)
+        for (long long i = k; i < r.S; i += stride) r.energy[i] = (double)r.efix[i] * kFixUnit;
+    if (k == 0) *r.error_out = *r.error;
 }
 
 }  // namespace
@@ -45,9 +57,14 @@ cudaError_t pack_walkers(const float* xyz, const int* n, int S, int nmax, const 
     return cudaGetLastError();
 }
 
-cudaError_t unpack_walkers(const float4* pos, long long count, int nmax, const int* n, float* xyz, cudaStream_t s) {
-    if (count == 0) return cudaSuccess;
-    unpack_walkers_kernel<<<(unsigned)((count + 255) / 256), 256, 0, s>>>(pos, count, nmax, n, xyz);
+cudaError_t read_back(const float4* pos, long long count, int nmax, const int* n, float* xyz, const ReadBack& r,
+                      cudaStream_t s) {
+    // a thread per position, or per word of a launch of at most 64 CTAs
+    long long most = r.energy ? r.S : 1;
+    for (int q = 0; q < ReadBack::kSegs; ++q) most = most > r.words[q] ? most : r.words[q];
+    long long ctas = (most + 255) / 256 < 64 ? (most + 255) / 256 : 64;
+    if (xyz && (count + 255) / 256 > ctas) ctas = (count + 255) / 256;
+    read_back_kernel<<<(unsigned)ctas, 256, 0, s>>>(pos, count, nmax, n, xyz, r);
     return cudaGetLastError();
 }
 
