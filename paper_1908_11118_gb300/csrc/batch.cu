@@ -266,14 +266,18 @@ regc_status regc_batch_create(regc_handle* const* handles, int count, int sweeps
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev);
     // size classes by (Nmax, sampling mode, cluster); within a class the largest systems first
-    std::map<std::tuple<int, int, int, int>, std::vector<int>> by_nmax;
-    for (int m = 0; m < count; ++m)
-        by_nmax[{handles[m]->nmax, b->member_da[m], handles[m]->P.n_cluster > 0 ? 1 : 0,
-                 sweep_direct(handles[m]->P) ? 1 : 0}].push_back(m);
+    std::map<std::tuple<int, int, int, int, int>, std::vector<int>> by_nmax;
+    for (int m = 0; m < count; ++m) {
+        const SweepParams& P = handles[m]->P;
+        const bool cl = P.n_cluster > 0;
+        by_nmax[{handles[m]->nmax, b->member_da[m], cl ? 1 : 0, sweep_direct(P) ? 1 : 0,
+                 sweep_geo(P) == 1 && !cl && !b->member_da[m] ? 1 : 0}].push_back(m);
+    }
     for (auto it = by_nmax.rbegin(); it != by_nmax.rend(); ++it) {
         Bucket q;
         q.nmax = std::get<0>(it->first);
-        q.c = BatchClass{std::get<1>(it->first) != 0, std::get<2>(it->first) != 0, std::get<3>(it->first) != 0};
+        q.c = BatchClass{std::get<1>(it->first) != 0, std::get<2>(it->first) != 0, std::get<3>(it->first) != 0,
+                         std::get<4>(it->first) != 0};
         std::vector<int> ms = it->second;
         q.members = ms;
         std::stable_sort(ms.begin(), ms.end(), [&](int a, int c) {

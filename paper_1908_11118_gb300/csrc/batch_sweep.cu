@@ -15,12 +15,13 @@ namespace {
 // systems of the launch sample with delayed acceptance (their networks'
 // fragments take ~240 registers per thread, so at most kBatchMaxWarpsDA
 // walkers per CTA); CL: every system of the launch carries a cluster species;
-// DIRECT: its walkers enumerate all particles instead of a cell list.
+// DIRECT: its walkers enumerate all particles instead of a cell list; SLAB:
+// every system of the launch is a rectangular slab (sweep_geo 1).
 constexpr int kBatchMaxWarps = 16;
 constexpr int kBatchMaxWarpsDA = 4;
 constexpr int kBatchHead = (int)((sizeof(SweepParams) + sizeof(int) + 15) / 16 * 16);   // parameters and item
 
-template <bool DA, bool CL, bool DIRECT, int K>
+template <bool DA, bool CL, bool DIRECT, bool SLAB, int K>
 __global__ void __launch_bounds__(32 * (DA ? kBatchMaxWarpsDA : kBatchMaxWarps))
     batch_sweep_kernel(const SweepParams* __restrict__ sys, const int2* __restrict__ items, int n_items,
                        int* counter, int region) {
@@ -46,7 +47,7 @@ __global__ void __launch_bounds__(32 * (DA ? kBatchMaxWarpsDA : kBatchMaxWarps))
         int* dst = reinterpret_cast<int*>(mine);
         for (int k = tid; k < (int)(sizeof(SweepParams) / sizeof(int)); k += 32 * K) dst[k] = src[k];
         group_sync<K>(bar);
-        walker_sweep<K, false, DA, CL, DIRECT>(Psh, mw.y, mine + kBatchHead, tid, bar);
+        walker_sweep<K, false, DA, CL, DIRECT, SLAB ? 1 : 0>(Psh, mw.y, mine + kBatchHead, tid, bar);
         group_sync<K>(bar);   // the slot and the item are rewritten for the next walker
     }
 }
@@ -74,10 +75,10 @@ struct Launch {
     int walkers_per_cta, grid, region;
     cudaStream_t s;
     cudaError_t err = cudaErrorInvalidValue;
-    template <bool DA, bool CL, bool DIRECT, int K>
+    template <bool DA, bool CL, bool DIRECT, bool SLAB, int K>
     void run() {
         const size_t smem = (size_t)walkers_per_cta * region;
-        batch_sweep_kernel<DA, CL, DIRECT, K>
+        batch_sweep_kernel<DA, CL, DIRECT, SLAB, K>
             <<<grid, 32 * K * walkers_per_cta, smem, s>>>(sys, items, n_items, counter, region);
         err = cudaGetLastError();
     }
@@ -86,10 +87,10 @@ struct Launch {
 struct Prepare {
     int max_smem;
     cudaError_t err = cudaSuccess;
-    template <bool DA, bool CL, bool DIRECT, int K>
+    template <bool DA, bool CL, bool DIRECT, bool SLAB, int K>
     void run() {
         if (err == cudaSuccess)
-            err = cudaFuncSetAttribute(batch_sweep_kernel<DA, CL, DIRECT, K>,
+            err = cudaFuncSetAttribute(batch_sweep_kernel<DA, CL, DIRECT, SLAB, K>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        max_smem);
     }
@@ -99,34 +100,36 @@ struct Occupancy {
     int walkers_per_cta;
     size_t smem;
     int n = 0;
-    template <bool DA, bool CL, bool DIRECT, int K>
+    template <bool DA, bool CL, bool DIRECT, bool SLAB, int K>
     void run() {
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_sweep_kernel<DA, CL, DIRECT, K>,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_sweep_kernel<DA, CL, DIRECT, SLAB, K>,
                                                           32 * K * walkers_per_cta, smem) != cudaSuccess)
             n = 0;
     }
 };
 
-// f.run<DA, CL, DIRECT, K>() of a class; false where there is no such kernel:
-// delayed acceptance follows the cell list, and more than one warp per walker
-// is for plain one-species walkers.
+// f.run<DA, CL, DIRECT, SLAB, K>() of a class; false where there is no such
+// kernel: delayed acceptance follows the cell list, more than one warp per
+// walker is for plain one-species walkers, and so is the slab's own form.
+template <int K, class F>
+void dispatch_plain(const BatchClass& c, F& f) {
+    if (c.direct && c.slab) f.template run<false, false, true, true, K>();
+    else if (c.direct) f.template run<false, false, true, false, K>();
+    else if (c.slab) f.template run<false, false, false, true, K>();
+    else f.template run<false, false, false, false, K>();
+}
+
 template <class F>
 bool dispatch(const BatchClass& c, int K, F& f) {
-    if (c.da && c.direct) return false;
-    if (K == 1) {
-        if (c.da && c.cl) f.template run<true, true, false, 1>();
-        else if (c.da) f.template run<true, false, false, 1>();
-        else if (c.cl && c.direct) f.template run<false, true, true, 1>();
-        else if (c.cl) f.template run<false, true, false, 1>();
-        else if (c.direct) f.template run<false, false, true, 1>();
-        else f.template run<false, false, false, 1>();
-        return true;
-    }
-    if (c.da || c.cl || (K != 2 && K != 4)) return false;
-    if (K == 2 && c.direct) f.template run<false, false, true, 2>();
-    else if (K == 2) f.template run<false, false, false, 2>();
-    else if (c.direct) f.template run<false, false, true, 4>();
-    else f.template run<false, false, false, 4>();
+    if ((c.da && c.direct) || ((c.da || c.cl) && (c.slab || K != 1))) return false;
+    if (c.da && c.cl) f.template run<true, true, false, false, 1>();
+    else if (c.da) f.template run<true, false, false, false, 1>();
+    else if (c.cl && c.direct) f.template run<false, true, true, false, 1>();
+    else if (c.cl) f.template run<false, true, false, false, 1>();
+    else if (K == 1) dispatch_plain<1>(c, f);
+    else if (K == 2) dispatch_plain<2>(c, f);
+    else if (K == 4) dispatch_plain<4>(c, f);
+    else return false;
     return true;
 }
 
@@ -145,8 +148,9 @@ cudaError_t launch_batch_sweep(const SweepParams* sys, const int2* items, int n_
 
 cudaError_t batch_prepare(int max_smem) {
     Prepare f{max_smem};
-    for (int bits = 0; bits < 8; ++bits)
-        for (int K = 1; K <= 4; K *= 2) dispatch(BatchClass{(bits & 1) != 0, (bits & 2) != 0, (bits & 4) != 0}, K, f);
+    for (int bits = 0; bits < 16; ++bits)
+        for (int K = 1; K <= 4; K *= 2)
+            dispatch(BatchClass{(bits & 1) != 0, (bits & 2) != 0, (bits & 4) != 0, (bits & 8) != 0}, K, f);
     return f.err;
 }
 

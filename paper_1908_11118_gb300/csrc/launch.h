@@ -31,6 +31,15 @@ inline int direct_limit(int ncell, long long walkers, int sms) {
 // cell list.
 inline bool sweep_direct(const SweepParams& P) { return P.direct && !P.delayed; }
 
+// The geometry the walk is compiled for (walker.cuh: make_hot): 1 a rectangular
+// cell and 2 a sheared one, not periodic in z, over a surface of one atom type;
+// 3 a rectangular box, periodic in z, without a surface; 0 any.
+inline int sweep_geo(const SweepParams& P) {
+    const bool sheared = P.g.shear != 0.0f;
+    if (!P.g.periodic_z && P.st.n_all > 0 && P.st.one_type >= 0) return sheared ? 2 : 1;
+    return P.g.periodic_z && P.st.n_all == 0 && !sheared ? 3 : 0;
+}
+
 // Shared-memory bytes of one walker of the sweep kernel with W warps.
 size_t sweep_smem(const SweepParams& P, int warps_per_walker);
 
@@ -85,9 +94,10 @@ bool batch_admits(const SweepParams& P);
 int batch_max_warps(bool da);
 
 // What the systems of one batch launch have in common: da, sampling with
-// delayed acceptance; cl, a cluster species; direct, sweep_direct.
+// delayed acceptance; cl, a cluster species; direct, sweep_direct; slab,
+// sweep_geo 1 (only where it is used: without da and cl).
 struct BatchClass {
-    bool da, cl, direct;
+    bool da, cl, direct, slab;
 };
 
 // Persistent sweep of items (system, walker) of the systems sys[] (device

@@ -32,16 +32,18 @@
 // that latency: all lanes hold the walk's state and decide together (no result
 // goes through shared memory with one warp per walker), the surface column is
 // requested before the mobile partners are evaluated, and the parameters used
-// in the loop are held in registers.  A move takes 572 warp instructions at 4.9
-// cycles each on the 1024-replica fcc(111) grid (ncu: 1.9 of them waiting for a
-// fixed latency, 1.0 for shared memory or a shuffle, 0.4 for a branch, 0.3 for
-// the instruction fetch); it took 645 at 5.3 with a committing thread fed
-// through shared memory and the draws made one move at a time.  Steps of ten
-// sweeps, before / after: 16 fcc(100) replicas 406 / 243 us with the walkers read
-// back, a hundred REGC steps of 160 A18 replicas 2.2 / 1.1 ms, 4096 clusters
-// 950 / 555 us, the 1024-replica grid 400 / 375 us.  With delayed acceptance the
-// code of the features stands once instead of six times and the kernel is no
-// longer bound by the instruction fetch: 1930 / 864 us.
+// in the loop are held in registers.  A move took 645 warp instructions at 5.3
+// cycles each on the 1024-replica fcc(111) grid with a committing thread fed
+// through shared memory and the draws made one move at a time; it took 572 at
+// 4.9 (ncu: 1.9 of them waiting for a fixed latency, 1.0 for shared memory or a
+// shuffle, 0.4 for a branch, 0.3 for the instruction fetch) without them, and
+// fewer since the geometry is compiled in (make_hot) and cells out of reach are
+// left out (stencil_list).  Steps of ten sweeps, before / after all of it: 16
+// fcc(100) replicas 406 / 192 us with the walkers read back, a hundred REGC steps
+// of 160 A18 replicas 2.2 / 0.88 ms, 4096 clusters 950 / 456 us, the 1024-replica
+// grid 400 / 322 us.  With delayed acceptance the code of the features stands
+// once instead of six times and the kernel is no longer bound by the instruction
+// fetch: 1930 / 804 us.
 #pragma once
 
 #include "cells.cuh"
@@ -105,8 +107,17 @@ struct Hot {
     PairTab gg, gA, gAB, ts, tsA;   // ts, tsA: the surface tables where the surface has one type
     float max_disp;
     int nmax, mps;
+    bool sheared;                   // false: x is Cartesian as it stands
+    float wx, wy, wz, reach2;       // cell widths; squared distance beyond which a cell holds no partner
 };
 
+// GEO (sweep_geo): 0 any geometry; 1 a rectangular cell and 2 a sheared one over
+// a surface of one type, walls along z; 3 a fully periodic box without a surface.
+// What the general form needs beside it is then known at compile time and drops
+// out.  A launch of ten sweeps, general form / this (with the cells out of reach
+// left out too, stencil_list): 1024 fcc(111) replicas 332 / 285 us (form 1), 1024
+// of two gases 308 / 271 (1), 160 A18 132 / 108 (2), 4096 clusters 508 / 416 (3).
+template <int GEO>
 __device__ __forceinline__ Hot make_hot(const SweepParams& P) {
     Hot H;
     H.g = P.g;
@@ -120,7 +131,29 @@ __device__ __forceinline__ Hot make_hot(const SweepParams& P) {
     H.max_disp = P.max_disp;
     H.nmax = P.nmax;
     H.mps = P.mps;
+    H.sheared = GEO == 0 || GEO == 2;
+    if (GEO == 1 || GEO == 2) {
+        H.g.periodic_z = 0;
+        H.st.one_type = 0;
+        H.st.n_all = 1;
+    }
+    if (GEO == 3) {
+        H.g.periodic_z = 1;
+        H.st.n_all = 0;
+    }
+    H.wx = 1.0f / H.cg.icx;
+    H.wy = 1.0f / H.cg.icy;
+    H.wz = 1.0f / H.cg.icz;
+    // well beyond the rounding of a coordinate, a cell index or a width
+    const float zs = H.g.periodic_z ? H.g.Lz : fabsf(H.g.z_lo) + fabsf(H.g.z_hi);
+    const float reach = H.g.rc * 1.001f + 2e-6f * (H.g.Lx + H.g.Ly + zs);
+    H.reach2 = reach * reach;
     return H;
+}
+
+// Cartesian x component of a displacement in the cell frame.
+__device__ __forceinline__ float cart(const Hot& H, float du, float dv) {
+    return H.sheared ? cart_dx(H.g, du, dv) : du;
 }
 
 // Pair tables of the moving particle's species against a partner of the first
@@ -139,8 +172,7 @@ __device__ __forceinline__ float pair_phi_sel(float dx, float dy, float dz, floa
                                               int& n_in, bool& overlap) {
     const float r2 = r2_of(dx, dy, dz);
     const bool in = use && r2 < rc2;
-    const float rr = in ? r2 : 1.0f;
-    const float s2 = __fdividef(t.sig2, rr);
+    const float s2 = __fdividef(t.sig2, r2);   // (what r2 out of range, or 0, makes of it is dropped)
     const float s6 = __fmul_rn(__fmul_rn(s2, s2), s2);
     const float phi = __fmul_rn(t.eps4, __fmaf_rn(s6, s6, -s6));
     n_in += in;
@@ -366,6 +398,7 @@ struct LaneCell {
     bool in;
     int wx, wy, wz;
     float sx, sy, sz;
+    float ax, ay, az, bx, by, bz;   // the gap to that cell from a point f beyond its own's lower corner: |b - a f| per axis
 };
 
 __device__ __forceinline__ LaneCell lane_cell(const Hot& H, int lane) {
@@ -380,6 +413,14 @@ __device__ __forceinline__ LaneCell lane_cell(const Hot& H, int lane) {
     l.sx = l.x < 0 ? -H.g.Lx : H.g.Lx;
     l.sy = l.y < 0 ? -H.g.Ly : H.g.Ly;
     l.sz = l.z < 0 ? -H.g.Lz : H.g.Lz;
+    // (in a sheared cell the gap along x is not a Cartesian distance: left out)
+    const bool x_gap = !H.sheared || H.g.shear == 0.f;
+    l.ax = x_gap ? fabsf((float)l.x) : 0.f;
+    l.bx = x_gap && l.x > 0 ? H.wx : 0.f;
+    l.ay = fabsf((float)l.y);
+    l.by = l.y > 0 ? H.wy : 0.f;
+    l.az = fabsf((float)l.z);
+    l.bz = l.z > 0 ? H.wz : 0.f;
     return l;
 }
 
@@ -388,9 +429,13 @@ __device__ __forceinline__ LaneCell lane_cell(const Hot& H, int lane) {
 // slot base + j is the slot of its j-th candidate while j stays in the entry.
 // A shift s > 0 is taken off the query, s < 0 off the partner (every shifted
 // operand is exact, Sterbenz, so a displacement is rounded once).  Returns the
-// candidates; cnt and excl are this lane's own cell's.
+// candidates; cnt and excl are this lane's own cell's.  NQ queries (0: every
+// cell is listed): a cell beyond reach of all of them is left out -- a third of
+// the candidates where cells are little wider than rc.
+template <int NQ>
 __device__ __forceinline__ int stencil_list(const Hot& H, const uint16_t* cnts, Cell3 c, LaneCell lc, int lane,
-                                            float4* st, int& cnt, int& excl) {
+                                            float4* st, int& cnt, int& excl, float q0x, float q0y, float q0z,
+                                            float q1x, float q1y, float q1z) {
     int ix = c.x + lc.x, iy = c.y + lc.y, iz = c.z + lc.z;
     const bool wx = (unsigned)ix >= (unsigned)H.cg.ncx, wy = (unsigned)iy >= (unsigned)H.cg.ncy;
     const bool wz = (unsigned)iz >= (unsigned)H.cg.ncz;
@@ -404,6 +449,17 @@ __device__ __forceinline__ int stencil_list(const Hot& H, const uint16_t* cnts, 
         sz = wz ? lc.sz : 0.f;
     } else {
         in = in && !wz;
+    }
+    if (NQ > 0) {
+        const float x0 = (float)c.x * H.wx, y0 = (float)c.y * H.wy;
+        const float z0 = fmaf((float)c.z, H.wz, H.g.periodic_z ? 0.f : H.g.z_lo);
+        auto gap2 = [&](float x, float y, float z) {
+            const float gx = fmaf(lc.ax, x0 - x, lc.bx), gy = fmaf(lc.ay, y0 - y, lc.by), gz = fmaf(lc.az, z0 - z, lc.bz);
+            return fmaf(gx, gx, fmaf(gy, gy, gz * gz));
+        };
+        float d2 = gap2(q0x, q0y, q0z);
+        if (NQ == 2) d2 = fminf(d2, gap2(q1x, q1y, q1z));
+        in = in && d2 < H.reach2;
     }
     const int cell = (iz * H.cg.ncy + iy) * H.cg.ncx + ix;
     cnt = in ? (int)cnts[cell] : 0;
@@ -444,7 +500,7 @@ __device__ __forceinline__ void mobile_cells(const Hot& H, const WalkerSmem& S, 
                                              int split, const MoveTabs& mt) {
     float4* st = S.stencil + warp * 32;
     int cnt, excl;
-    const int total = stencil_list(H, S.cnt, c, lc, lane, st, cnt, excl);
+    const int total = stencil_list<NQ>(H, S.cnt, c, lc, lane, st, cnt, excl, q0x, q0y, q0z, q1x, q1y, q1z);
     bool ov = false, ov1 = false;
     int started = 0;
 #pragma unroll 2   // two batches' independent chains may overlap
@@ -458,19 +514,21 @@ __device__ __forceinline__ void mobile_cells(const Hot& H, const WalkerSmem& S, 
         const bool use = act && pj != skip;
         // lanes without a partner read particle 0 and discard the term
         const float4 p = S.pos[use ? pj : 0];
-        const float bx = __fsub_rn(p.x, fmaxf(-e.y, 0.f)), by = __fsub_rn(p.y, fmaxf(-e.z, 0.f)),
-                    bz = __fsub_rn(p.z, fmaxf(-e.w, 0.f));
-        const float ax = fmaxf(e.y, 0.f), ay = fmaxf(e.z, 0.f), az = fmaxf(e.w, 0.f);
+        const float bx = __fsub_rn(p.x, fmaxf(-e.y, 0.f)), by = __fsub_rn(p.y, fmaxf(-e.z, 0.f));
+        const float ax = fmaxf(e.y, 0.f), ay = fmaxf(e.z, 0.f);
+        const float bz = H.g.periodic_z ? __fsub_rn(p.z, fmaxf(-e.w, 0.f)) : p.z;
+        const float az0 = H.g.periodic_z ? __fsub_rn(q0z, fmaxf(e.w, 0.f)) : q0z;
         n_cand += use ? NQ : 0;
         const PairTab& tp = CL ? (pj < split ? mt.tA : mt.tB) : H.gg;
         const float dy0 = __fsub_rn(__fsub_rn(q0y, ay), by);
-        const float phi0 = pair_phi_sel(cart_dx(H.g, __fsub_rn(__fsub_rn(q0x, ax), bx), dy0), dy0,
-                                        __fsub_rn(__fsub_rn(q0z, az), bz), H.g.rc2, tp, use, n_in, ov);
+        const float phi0 = pair_phi_sel(cart(H, __fsub_rn(__fsub_rn(q0x, ax), bx), dy0), dy0,
+                                        __fsub_rn(az0, bz), H.g.rc2, tp, use, n_in, ov);
         fix_add(acc, phi0, 1);
         if (NQ == 2) {
+            const float az1 = H.g.periodic_z ? __fsub_rn(q1z, fmaxf(e.w, 0.f)) : q1z;
             const float dy1 = __fsub_rn(__fsub_rn(q1y, ay), by);
-            const float phi1 = pair_phi_sel(cart_dx(H.g, __fsub_rn(__fsub_rn(q1x, ax), bx), dy1), dy1,
-                                            __fsub_rn(__fsub_rn(q1z, az), bz), H.g.rc2, tp, use, n_in, ov1);
+            const float phi1 = pair_phi_sel(cart(H, __fsub_rn(__fsub_rn(q1x, ax), bx), dy1), dy1,
+                                            __fsub_rn(az1, bz), H.g.rc2, tp, use, n_in, ov1);
             fix_add(acc, phi1, -1);
         }
         started += __popc(starts);
@@ -506,13 +564,13 @@ __device__ __forceinline__ void mobile_direct(const Hot& H, const WalkerSmem& S,
         const PairTab& tp = CL ? (j < split ? mt.tA : mt.tB) : H.gg;
         const float dy0 = near_diff(q0y, p.y, H.g.Ly, H.g.hLy);
         const float dz0 = H.g.periodic_z ? near_diff(q0z, p.z, H.g.Lz, H.g.hLz) : __fsub_rn(q0z, p.z);
-        const float phi0 = pair_phi_sel(cart_dx(H.g, near_diff(q0x, p.x, H.g.Lx, H.g.hLx), dy0), dy0, dz0, H.g.rc2,
+        const float phi0 = pair_phi_sel(cart(H, near_diff(q0x, p.x, H.g.Lx, H.g.hLx), dy0), dy0, dz0, H.g.rc2,
                                         tp, use, n_in, ov);
         fix_add(acc, phi0, 1);
         if (NQ == 2) {
             const float dy1 = near_diff(q1y, p.y, H.g.Ly, H.g.hLy);
             const float dz1 = H.g.periodic_z ? near_diff(q1z, p.z, H.g.Lz, H.g.hLz) : __fsub_rn(q1z, p.z);
-            const float phi1 = pair_phi_sel(cart_dx(H.g, near_diff(q1x, p.x, H.g.Lx, H.g.hLx), dy1), dy1, dz1,
+            const float phi1 = pair_phi_sel(cart(H, near_diff(q1x, p.x, H.g.Lx, H.g.hLx), dy1), dy1, dz1,
                                             H.g.rc2, tp, use, n_in, ov1);
             fix_add(acc, phi1, -1);
         }
@@ -536,10 +594,9 @@ __device__ __forceinline__ void surface_diff(const Hot& H, float4 a, float qx, f
                                              float& dy, float& dz) {
     const unsigned bits = __float_as_uint(a.w);
     const float sx = (bits & 4u) ? H.g.Lx : 0.f, sy = (bits & 8u) ? H.g.Ly : 0.f;
-    const float sz = (bits & 16u) ? H.g.Lz : 0.f;
     dy = __fsub_rn(__fsub_rn(qy, sy), a.y);
-    dx = cart_dx(H.g, __fsub_rn(__fsub_rn(qx, sx), a.x), dy);
-    dz = __fsub_rn(__fsub_rn(qz, sz), a.z);
+    dx = cart(H, __fsub_rn(__fsub_rn(qx, sx), a.x), dy);
+    dz = __fsub_rn(H.g.periodic_z ? __fsub_rn(qz, (bits & 16u) ? H.g.Lz : 0.f) : qz, a.z);
 }
 
 template <bool CL>
@@ -584,7 +641,8 @@ __device__ __forceinline__ void query_features(const SweepParams& P, const Hot& 
                                                int warp, int split, const MoveTabs& mt) {
     float4* st = S.stencil + warp * 32;
     int cnt, excl;
-    const int total = stencil_list(H, S.cnt, cell3_hot(H, qx, qy, qz), lc, lane, st, cnt, excl);
+    const int total = stencil_list<0>(H, S.cnt, cell3_hot(H, qx, qy, qz), lc, lane, st, cnt, excl, 0.f, 0.f, 0.f, 0.f,
+                                      0.f, 0.f);
     const int n_mob = (total + 31) & ~31;
     const bool surf = near_surf(H, qz);
     const int n_all = n_mob + (surf ? H.st.stride : 0);
@@ -606,7 +664,7 @@ __device__ __forceinline__ void query_features(const SweepParams& P, const Hot& 
                     const float dy = __fsub_rn(__fsub_rn(qy, fmaxf(e.z, 0.f)), __fsub_rn(p.y, fmaxf(-e.z, 0.f)));
                     const float du = __fsub_rn(__fsub_rn(qx, fmaxf(e.y, 0.f)), __fsub_rn(p.x, fmaxf(-e.y, 0.f)));
                     const float dz = __fsub_rn(__fsub_rn(qz, fmaxf(e.w, 0.f)), __fsub_rn(p.z, fmaxf(-e.w, 0.f)));
-                    r2 = r2_of(cart_dx(H.g, du, dy), dy, dz);
+                    r2 = r2_of(cart(H, du, dy), dy, dz);
                     wgt = CL ? (pj < split ? mt.tA.eps : mt.tB.eps) : H.gg.eps;
                 }
             }
@@ -1093,12 +1151,12 @@ __device__ __forceinline__ int commit_move(const SweepParams& P, const Hot& H, c
 // n_sweeps sweeps of walker w by a group of K warps (tid: thread index in the
 // group, smem: the group's shared-memory region, bar: the group's named
 // barrier when K > 1).
-template <int K, bool TRACE, bool DA, bool CL, bool DIRECT>
+template <int K, bool TRACE, bool DA, bool CL, bool DIRECT, int GEO>
 __device__ __forceinline__ void walker_sweep(const SweepParams& P, int w, char* smem, int tid, int bar) {
     static_assert(!(DA && DIRECT), "the feature sums follow the cell list's order");
     const int lane = tid & 31, warp = tid >> 5;
     const WalkerSmem S = carve<K, DIRECT>(smem, P);
-    const Hot H = make_hot(P);
+    const Hot H = make_hot<GEO>(P);
 
     Walk W;
     W.N = P.n[w];
