@@ -9,18 +9,18 @@ namespace regc {
 
 // Nmax up to which a walker's moves enumerate every particle (walker.cuh).  A
 // stencil of 27 of the ncell cells spares the share 1 - 27 / ncell of the
-// distances and costs what about 52 of them do; with many walkers per SM the
+// distances and costs what about 96 of them do; with many walkers per SM the
 // smaller region counts too (more of them resident), and the line lies higher.
 // Microseconds of a ten-sweep launch, direct / cells, every walker nearly full:
-//   fcc(111), 168 cells, 16 walkers:   137 / 157 at Nmax 32, 158 / 158 at 64, 172 / 161 at 96
-//   periodic cube, 125 cells, 16 walkers:   167 / 192 at 20, 236 / 200 at 68
-//   periodic cube, 4096 walkers (27 per SM):   391 / 493 at 20, 578 / 640 at 68,
-//     652 / 683 at 128, 729 / 747 at 160, 809 / 782 at 192
-//   A18, 40 cells, 160 walkers of 20 particles:   88 / 105
+//   fcc(111), 168 cells, 16 walkers:   136 / 152 at Nmax 64, 144 / 153 at 96, 148 / 157 at 128, 159 / 157 at 192
+//   fcc(111), 1024 walkers (7 per SM):   184 / 207 at 64, 203 / 210 at 96, 218 / 212 at 128
+//   periodic cube, 125 cells, 16 walkers:   160 / 165 at 68, 164 / 172 at 96, 178 / 176 at 128
+//   periodic cube, 4096 walkers (27 per SM):   416 / 544 at 68, 475 / 551 at 128, 533 / 564 at 160, 593 / 583 at 192
+//   A18, 40 cells, 160 walkers of 20 particles:   78 / 101
 constexpr int kDirectMax = 160;
 
 inline int direct_limit(int ncell, long long walkers, int sms) {
-    const int line = walkers > 12LL * sms ? kDirectMax : 52;
+    const int line = walkers > 12LL * sms ? kDirectMax : 96;
     if (ncell <= 27) return kDirectMax;
     const long long n = (long long)line * ncell / (ncell - 27);
     return n < kDirectMax ? (int)n : kDirectMax;

@@ -70,10 +70,10 @@ def two_gas(nmax):
     return p, pos, n, (n // 2).astype(np.int32)
 
 
-# the largest Nmax of the direct enumeration: 160, or 52 ncell / (ncell - 27)
+# the largest Nmax of the direct enumeration: 160, or 96 ncell / (ncell - 27)
 # with few walkers per SM and more than 27 cells (168 and 125 here)
-@pytest.mark.parametrize("system,limit", [(fcc111, 61), (fcc100, 160), (minimal_periods, 160), (hexagonal, 160),
-                                          (cluster, 66), (cluster_many, 160), (two_gas, 160)])
+@pytest.mark.parametrize("system,limit", [(fcc111, 114), (fcc100, 160), (minimal_periods, 160), (hexagonal, 160),
+                                          (cluster, 122), (cluster_many, 160), (two_gas, 160)])
 @pytest.mark.parametrize("warps", [1, 2, 4])
 def test_direct_and_cells_make_the_same_moves(system, limit, warps, monkeypatch):
     monkeypatch.setenv("REGC_WARPS_PER_WALKER", str(warps))
