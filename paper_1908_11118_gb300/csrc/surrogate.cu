@@ -670,36 +670,59 @@ __device__ __forceinline__ void adam_update(float g, float c1, float c2, float l
     theta -= lr * mh / (sqrtf(vh) + eps);
 }
 
-// Many training steps in one launch: a cluster of one CTA per 128 rows of the
-// mini-batch (at most eight), each with a copy of the operands in shared
-// memory.  Per step: the gradient of the CTA's rows into its shared memory; the
-// cluster meets; CTA r adds the CTAs' gradients of its share of the parameters
-// through distributed shared memory, in CTA order, takes their Adam step (the
-// FP32 masters and moments of its share stay in its shared memory) and writes
-// the new operands into every CTA's copy; the cluster meets again.  The rows of
-// the next step are drawn (Philox stream 6) and requested while this one runs.
+// Many training steps in one launch: a cluster of eight CTAs, each with a copy
+// of the operands in shared memory and up to 128 rows of the mini-batch (the
+// first CTAs that the batch fills; the others have none).  Per step: the
+// gradient of the CTA's rows into its shared memory; the cluster meets; CTA r
+// adds the CTAs' gradients of its eighth of the parameters through distributed
+// shared memory, in CTA order, takes their Adam step (the FP32 masters and
+// moments of its share stay in its shared memory) and writes the new operands
+// into every CTA's copy; the cluster meets again.  The rows of the next step
+// are drawn (Philox stream 6) and requested while this one runs.
 //
-// A step is one chain of dependent pieces, so what counts is its latency, and
-// what makes it up are the SiLUs and their derivatives of 128 x 128 units by
-// few warps.  Eight warps share them: warps w and w + 4 take the same 32 rows,
-// one the lower half of each layer's units, the other the upper, and pass each
-// other the A fragments (and the running output sum) through shared memory.
-// Every sum keeps the terms and the order it has in tc_gradient, hence its
-// bits.
-constexpr int kMaxTrainCtas = 8;   // the portable cluster size
+// A step is one chain of dependent pieces, so what counts is its latency.
+// Eight warps share it: warps w and w + 4 take the same 32 rows, one the lower
+// half of each layer's units, the other the upper, and pass each other the A
+// fragments (and the running output sum) through shared memory.  Every sum
+// keeps the terms and the order it has in tc_gradient, hence its bits.
+//   - Operands and tiles lie row-major and are read with ldmatrix, transposed
+//     where a product contracts over the rows: one copy of each, written in
+//     whole words, instead of a second one written half-word by half-word.
+//   - A parameter update is pushed to the other CTAs two parameters a store,
+//     next to its neighbours'; scattered half-words to two copies each, with
+//     the loss collected by one thread, took 12600 of a step's 33000 cycles.
+//   - The derivatives of the SiLUs take one branch for 32 values instead of one
+//     a reciprocal (dsilu_all); they were most of 10600 cycles.
+//   - The next rows are drawn, and the next step's bias corrections taken, while
+//     the cluster's barrier is waited for.
+// A step of 1024 rows takes 9.0 us (16.3 before these), of 512 8.6 (16.1), of 128
+// 8.6 (18.7, with a cluster of one CTA per 128 rows); a quarter of it is the MUFU
+// unit's on the SiLUs, a third the two barriers and the update between them.
+constexpr int kTrainCtas = 8;   // the portable cluster size
 constexpr int kXLd = kNF + 4;      // padded row of the staged features
 constexpr int kTrainThreads = 2 * kTcRows;
+constexpr int kPairs = (kNParams + 1) / 2;
+constexpr int kShare = (kPairs + kTrainCtas - 1) / kTrainCtas;   // of each CTA, in pairs
 
 struct TrainSmem {
-    TcSmem tc;
+    // operands and tiles; their rows are 12 and 36 words apart, so that the
+    // eight rows of an ldmatrix lie in different banks
+    __nv_bfloat16 w1[kNF][kTcLd2];     // W1 [k][u]
+    __nv_bfloat16 w2[kNH][kTcLd2];     // W2 [u][v]
+    __nv_bfloat16 xb[kTcRows][kTcLd1]; // bf(X)
+    __nv_bfloat16 h1[kTcRows][kTcLd2]; // bf(h1)
+    __nv_bfloat16 d2[kTcRows][kTcLd2]; // bf(dz2)
+    __nv_bfloat16 d1[kTcRows][kTcLd2]; // bf(dz1)
+    float w3[kNH], b1[kNH], b2[kNH];
+    float b3[2], pad[2], loss[kTrainCtas];   // loss: the CTAs' sums, in the first CTA
     float grad[kNParams + 3];
-    float loss, pad[3];
     float x[2][kTcRows][kXLd];
     float y[2][kTcRows];
-    uint32_t xch[kTcWarps][2][16][32];   // A fragments of the two halves' units, by pair of warps
-    float o[kTcWarps][4][32];            // running output sums of the lower halves
-    float e[kTcWarps][4][32];            // outputs
-    float own[1];              // [3][share]: theta, m, v of this CTA's share
+    float red[kTcWarps][3][kNH];       // per-pair sums over rows: dW3, db2, db1
+    float red_s[kTcWarps][2];          // per-pair db3, squared residuals
+    float o[kTcWarps][4][32];          // running output sums of the lower halves
+    float e[kTcWarps][4][32];          // outputs
+    float2 own_t[kShare], own_m[kShare], own_v[kShare];   // theta, m, v of this CTA's share
 };
 
 // Barrier of the two warps of a pair.
@@ -707,93 +730,170 @@ __device__ __forceinline__ void pair_sync(int pair) {
     asm volatile("bar.sync %0, 64;" ::"r"(1 + pair) : "memory");
 }
 
-// Write this half's A words into the pair's exchange and its transposed copy.
-__device__ __forceinline__ void share_frag(uint32_t (*xch)[32], __nv_bfloat16 (*tr)[kTcLd],
-                                           const uint32_t (&own)[2][2][4], int pair, int half, int lane) {
+// The two halves of the cluster's barrier.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// Four 8 x 8 matrices, lane l giving the address of row l % 8 of matrix l / 8.
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p))
+                 : "memory");
+}
+
+__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], const __nv_bfloat16* p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p))
+                 : "memory");
+}
+
+// 1 / d rounded to nearest, for 1 <= d < 2^117: the correction of a reciprocal
+// within one ulp by its exact residual (P. Markstein, IBM J. Res. Dev. 34,
+// 1990).  Equal to the division for each of those numbers (all of them were
+// compared), without its branch.
+__device__ __forceinline__ float reciprocal(float d) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return fmaf(r, fmaf(-d, r, 1.0f), r);
+}
+
+// z <- silu'(z) of a lane's 32 values, as dsilu_f.
+__device__ __forceinline__ void dsilu_all(float (&z)[2][4][4]) {
+    bool far = false;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) far |= !(z[k >> 4][(k >> 2) & 3][k & 3] > -80.f);
+    if (__any_sync(FULL, far)) {
+#pragma unroll 1
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                float& x = mt ? z[1][k >> 2][k & 3] : z[0][k >> 2][k & 3];
+                x = dsilu_f(x);
+            }
+        return;
+    }
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        float& x = z[k >> 4][(k >> 2) & 3][k & 3];
+        const float s = reciprocal(1.0f + expf(-x));
+        x = s * (1.0f + x * (1.0f - s));
+    }
+}
+
+// Where parameters i and i + 1 (i even) lie among the operands: a pair of bf16
+// or of floats (the last parameter, b3, takes its pad along).
+struct OperandPair {
+    void* at;
+    bool half;
+};
+__device__ __forceinline__ OperandPair operand_pair(TrainSmem& sm, int i) {
+    constexpr int o1 = kNF * kNH, o2 = o1 + kNH, o3 = o2 + kNH * kNH, o4 = o3 + kNH, o5 = o4 + kNH;
+    static_assert(o5 % 2 == 0 && kNH % 2 == 0, "a pair lies within one array");
+    if (i < o1) return {&sm.w1[i / kNH][i % kNH], true};
+    if (i < o2) return {&sm.b1[i - o1], false};
+    if (i < o3) return {&sm.w2[(i - o2) / kNH][(i - o2) % kNH], true};
+    if (i < o4) return {&sm.b2[i - o3], false};
+    if (i < o5) return {&sm.w3[i - o4], false};
+    return {sm.b3, false};
+}
+__device__ __forceinline__ void store_operands(OperandPair p, float2 v) {
+    if (p.half) *reinterpret_cast<uint32_t*>(p.at) = pack_bf16(v.x, v.y);
+    else *reinterpret_cast<float2*>(p.at) = v;
+}
+
+// A fragments own (this half's units) into rows 32 pair .. of tile m.
+__device__ __forceinline__ void store_frag(__nv_bfloat16 (*m)[kTcLd2], const uint32_t (&own)[2][2][4], int pair,
+                                           int half, int lane) {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-        for (int kh = 0; kh < 2; ++kh) {
-            const uint32_t(&r)[4] = own[mt][kh];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) xch[8 * mt + 4 * kh + q][lane] = r[q];
-            const int rg = pair * 32 + 16 * mt + g, u = 16 * (2 * half + kh) + 2 * t;
-            const __nv_bfloat162 a0 = *reinterpret_cast<const __nv_bfloat162*>(&r[0]);
-            const __nv_bfloat162 a1 = *reinterpret_cast<const __nv_bfloat162*>(&r[1]);
-            const __nv_bfloat162 a2 = *reinterpret_cast<const __nv_bfloat162*>(&r[2]);
-            const __nv_bfloat162 a3 = *reinterpret_cast<const __nv_bfloat162*>(&r[3]);
-            tr[u][rg] = a0.x;     tr[u + 1][rg] = a0.y;
-            tr[u][rg + 8] = a1.x; tr[u + 1][rg + 8] = a1.y;
-            tr[u + 8][rg] = a2.x; tr[u + 9][rg] = a2.y;
-            tr[u + 8][rg + 8] = a3.x; tr[u + 9][rg + 8] = a3.y;
-        }
-}
-
-// The A fragments of all units from this half's and the partner's.
-__device__ __forceinline__ void gather_frag(const uint32_t (*other)[32], const uint32_t (&own)[2][2][4], int half,
-                                            int lane, uint32_t (&a)[2][4][4]) {
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
         for (int kh = 0; kh < 2; ++kh)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t x = other[8 * mt + 4 * kh + q][lane];
-                a[mt][kh][q] = half ? x : own[mt][kh][q];
-                a[mt][2 + kh][q] = half ? own[mt][kh][q] : x;
-            }
+            for (int q = 0; q < 4; ++q)
+                *reinterpret_cast<uint32_t*>(
+                    &m[pair * 32 + 16 * mt + g + 8 * (q & 1)][16 * (2 * half + kh) + 8 * (q >> 1) + 2 * t]) =
+                    own[mt][kh][q];
+}
+
+// Sums over the 8 lane groups (g) of eight values, as sum_over_g adds them: each
+// lane ends with one of the totals, that of index 4 g0 + 2 g1 + g2 by the bits of
+// its g (7 exchanges instead of 24).
+__device__ __forceinline__ float sums_over_g(const float (&v)[4][2], int lane) {
+    float a[4], b[2];
+    const bool g0 = lane & 4, g1 = lane & 8, g2 = lane & 16;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float lo = v[i >> 1][i & 1], hi = v[2 + (i >> 1)][i & 1];
+        a[i] = (g0 ? hi : lo) + __shfl_xor_sync(FULL, g0 ? lo : hi, 4);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) b[i] = (g1 ? a[2 + i] : a[i]) + __shfl_xor_sync(FULL, g1 ? a[i] : a[2 + i], 8);
+    return (g2 ? b[1] : b[0]) + __shfl_xor_sync(FULL, g2 ? b[0] : b[1], 16);
 }
 
 // tc_gradient by eight warps: this CTA's gradient into sm.grad, its sum of
-// squared residuals into sm.loss.
-__device__ __forceinline__ void train_gradient(TrainSmem& ts, const uint32_t (&ax)[2][4], const bool (&act)[2][2],
-                                               const float (&y)[2][2], float scale, int tid) {
-    TcSmem& sm = ts.tc;
+// squared residuals into *loss.
+__device__ __forceinline__ void train_gradient(TrainSmem& sm, const uint32_t (&ax)[2][4], const bool (&act)[2][2],
+                                               const float (&y)[2][2], float scale, float* loss, int tid) {
     const int lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
     const int pair = warp & 3, half = warp >> 2;
-    __syncthreads();   // the operands and the transposed rows
-    // forward, layer 1: this half's units 8 (4 half + jj) ..
+    const int l15 = lane & 15, l8 = 8 * (lane >> 4);   // ldmatrix: row and column of a 16 x 16 tile
+    const int m15 = (lane & 7) + 8 * (lane >> 4), m8 = 8 * ((lane >> 3) & 1);   // its middle matrices exchanged
+    // forward, layer 1: this half's units 32 half + 8 jj ..
     float z1[2][4][4];
     uint32_t own[2][2][4], a[2][4][4];
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
+    for (int kh = 0; kh < 2; ++kh) {
+        uint32_t b[4];
+        ldsm4_t(b, &sm.w1[l15][32 * half + 16 * kh + l8]);
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            const int j = 4 * half + jj, u = 8 * j + 2 * t;
-            z1[mt][jj][0] = z1[mt][jj][2] = sm.b1[u];
-            z1[mt][jj][1] = z1[mt][jj][3] = sm.b1[u + 1];
-            const uint32_t b[2] = {lds_u32(&sm.w1u[8 * j + g][2 * t]), lds_u32(&sm.w1u[8 * j + g][2 * t + 8])};
-            mma_bf16(z1[mt][jj], ax[mt], b);
-        }
-#pragma unroll
-        for (int kh = 0; kh < 2; ++kh)
+        for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                const float* c = z1[mt][2 * kh + q];
+                const int u = 32 * half + 16 * kh + 8 * q + 2 * t;
+                float(&c)[4] = z1[mt][2 * kh + q];
+                c[0] = c[2] = sm.b1[u];
+                c[1] = c[3] = sm.b1[u + 1];
+                const uint32_t bq[2] = {b[2 * q], b[2 * q + 1]};
+                mma_bf16(c, ax[mt], bq);
                 own[mt][kh][2 * q] = pack_bf16(silu_f(c[0]), silu_f(c[1]));
                 own[mt][kh][2 * q + 1] = pack_bf16(silu_f(c[2]), silu_f(c[3]));
             }
     }
-    share_frag(ts.xch[pair][half], sm.h1t, own, pair, half, lane);
+    store_frag(sm.h1, own, pair, half, lane);
     pair_sync(pair);
-    gather_frag(ts.xch[pair][half ^ 1], own, half, lane, a);
-    // forward, layer 2
-    float z2[2][4][4];
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            const int j = 4 * half + jj, v = 8 * j + 2 * t;
-            z2[mt][jj][0] = z2[mt][jj][2] = sm.b2[v];
-            z2[mt][jj][1] = z2[mt][jj][3] = sm.b2[v + 1];
+        for (int kk = 0; kk < 4; ++kk) ldsm4(a[mt][kk], &sm.h1[pair * 32 + 16 * mt + l15][16 * kk + l8]);
+    // forward, layer 2
+    float z2[2][4][4];
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                const uint32_t b[2] = {lds_u32(&sm.w2u[8 * j + g][16 * kk + 2 * t]),
-                                       lds_u32(&sm.w2u[8 * j + g][16 * kk + 2 * t + 8])};
-                mma_bf16(z2[mt][jj], a[mt][kk], b);
+    for (int kh = 0; kh < 2; ++kh) {
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int v = 32 * half + 16 * kh + 8 * q + 2 * t;
+                z2[mt][2 * kh + q][0] = z2[mt][2 * kh + q][2] = sm.b2[v];
+                z2[mt][2 * kh + q][1] = z2[mt][2 * kh + q][3] = sm.b2[v + 1];
             }
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) {
+            uint32_t b[4];
+            ldsm4_t(b, &sm.w2[16 * kk + l15][32 * half + 16 * kh + l8]);
+#pragma unroll
+            for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const uint32_t bq[2] = {b[2 * q], b[2 * q + 1]};
+                    mma_bf16(z2[mt][2 * kh + q], a[mt][kk], bq);
+                }
         }
+    }
     // the output: the lower half's units first, then the upper's
     float s2[2][4][4];
 #pragma unroll
@@ -804,9 +904,10 @@ __device__ __forceinline__ void train_gradient(TrainSmem& ts, const uint32_t (&a
             for (int c = 0; c < 4; ++c) s2[mt][jj][c] = silu_f(z2[mt][jj][c]);
     float o[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, e[2][2];
     if (half) {
+        dsilu_all(z2);   // (while the lower half adds its units)
         pair_sync(pair);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) o[q >> 1][q & 1] = ts.o[pair][q][lane];
+        for (int q = 0; q < 4; ++q) o[q >> 1][q & 1] = sm.o[pair][q][lane];
     }
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
@@ -816,18 +917,6 @@ __device__ __forceinline__ void train_gradient(TrainSmem& ts, const uint32_t (&a
             o[mt][0] = fmaf(s2[mt][jj][0], sm.w3[v], fmaf(s2[mt][jj][1], sm.w3[v + 1], o[mt][0]));
             o[mt][1] = fmaf(s2[mt][jj][2], sm.w3[v], fmaf(s2[mt][jj][3], sm.w3[v + 1], o[mt][1]));
         }
-    if (!half) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) ts.o[pair][q][lane] = o[q >> 1][q & 1];
-        pair_sync(pair);
-    }
-    // meanwhile: the derivatives
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) z2[mt][jj][c] = dsilu_f(z2[mt][jj][c]);
     if (half) {
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
@@ -837,14 +926,19 @@ __device__ __forceinline__ void train_gradient(TrainSmem& ts, const uint32_t (&a
                 float x = o[mt][h];
                 x += __shfl_xor_sync(FULL, x, 1);
                 x += __shfl_xor_sync(FULL, x, 2);
-                e[mt][h] = x + sm.b3;
-                ts.e[pair][2 * mt + h][lane] = e[mt][h];
+                e[mt][h] = x + sm.b3[0];
+                sm.e[pair][2 * mt + h][lane] = e[mt][h];
             }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sm.o[pair][q][lane] = o[q >> 1][q & 1];
+        pair_sync(pair);
+        dsilu_all(z2);   // (while the upper half adds its own)
     }
     pair_sync(pair);
     if (!half) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) e[q >> 1][q & 1] = ts.e[pair][q][lane];
+        for (int q = 0; q < 4; ++q) e[q >> 1][q & 1] = sm.e[pair][q][lane];
     }
     // residuals and d loss / d e
     float ge[2][2], sq = 0.f, gsum = 0.f;
@@ -886,147 +980,121 @@ __device__ __forceinline__ void train_gradient(TrainSmem& ts, const uint32_t (&a
                 own[mt][kh][2 * q + 1] = pack_bf16(c[2], c[3]);
             }
     }
-    share_frag(ts.xch[pair][half], sm.d2t, own, pair, half, lane);
+    store_frag(sm.d2, own, pair, half, lane);
+    dsilu_all(z1);
+    pair_sync(pair);
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) z1[mt][jj][c] = dsilu_f(z1[mt][jj][c]);
-    pair_sync(pair);
-    gather_frag(ts.xch[pair][half ^ 1], own, half, lane, a);
+        for (int kk = 0; kk < 4; ++kk) ldsm4(a[mt][kk], &sm.d2[pair * 32 + 16 * mt + l15][16 * kk + l8]);
     // backward through layer 2
     float db1[4][2];
 #pragma unroll
     for (int jj = 0; jj < 4; ++jj) db1[jj][0] = db1[jj][1] = 0.f;
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
+    for (int kh = 0; kh < 2; ++kh) {
+        float c[2][2][4] = {};
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            const int j = 4 * half + jj;
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int kk = 0; kk < 4; ++kk) {
+            uint32_t b[4];
+            ldsm4(b, &sm.w2[32 * half + 16 * kh + m15][16 * kk + m8]);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                const uint32_t b[2] = {lds_u32(&sm.w2r[8 * j + g][16 * kk + 2 * t]),
-                                       lds_u32(&sm.w2r[8 * j + g][16 * kk + 2 * t + 8])};
-                mma_bf16(c, a[mt][kk], b);
-            }
+            for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float d = c[q] * z1[mt][jj][q];
-                z1[mt][jj][q] = d;
-                db1[jj][q & 1] += d;
-            }
+                for (int q = 0; q < 2; ++q) {
+                    const uint32_t bq[2] = {b[2 * q], b[2 * q + 1]};
+                    mma_bf16(c[mt][q], a[mt][kk], bq);
+                }
         }
 #pragma unroll
-        for (int kh = 0; kh < 2; ++kh)
+        for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                const float* c = z1[mt][2 * kh + q];
-                own[mt][kh][2 * q] = pack_bf16(c[0], c[1]);
-                own[mt][kh][2 * q + 1] = pack_bf16(c[2], c[3]);
+                const int jj = 2 * kh + q;
+                float d[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    d[i] = c[mt][q][i] * z1[mt][jj][i];
+                    db1[jj][i & 1] += d[i];
+                }
+                own[mt][kh][2 * q] = pack_bf16(d[0], d[1]);
+                own[mt][kh][2 * q + 1] = pack_bf16(d[2], d[3]);
             }
     }
-    // (the exchange is read by the partner up to its own writes here, so the
-    // transposed copy alone is written)
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int kh = 0; kh < 2; ++kh) {
-            const uint32_t(&r)[4] = own[mt][kh];
-            const int rg = pair * 32 + 16 * mt + g, u = 16 * (2 * half + kh) + 2 * t;
-            const __nv_bfloat162 a0 = *reinterpret_cast<const __nv_bfloat162*>(&r[0]);
-            const __nv_bfloat162 a1 = *reinterpret_cast<const __nv_bfloat162*>(&r[1]);
-            const __nv_bfloat162 a2 = *reinterpret_cast<const __nv_bfloat162*>(&r[2]);
-            const __nv_bfloat162 a3 = *reinterpret_cast<const __nv_bfloat162*>(&r[3]);
-            sm.d1t[u][rg] = a0.x;     sm.d1t[u + 1][rg] = a0.y;
-            sm.d1t[u][rg + 8] = a1.x; sm.d1t[u + 1][rg + 8] = a1.y;
-            sm.d1t[u + 8][rg] = a2.x; sm.d1t[u + 9][rg] = a2.y;
-            sm.d1t[u + 8][rg + 8] = a3.x; sm.d1t[u + 9][rg + 8] = a3.y;
-        }
-    // per-warp sums over rows of dW3, db2, db1, db3 and the squared residuals
-#pragma unroll
-    for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const float s3 = sum_over_g(dw3[jj][q]), sb2 = sum_over_g(db2[jj][q]), sb1 = sum_over_g(db1[jj][q]);
-            if (g == 0) {
-                const int u = 8 * (4 * half + jj) + 2 * t + q;
-                sm.red[pair][0][u] = s3;
-                sm.red[pair][1][u] = sb2;
-                sm.red[pair][2][u] = sb1;
-            }
-        }
+    store_frag(sm.d1, own, pair, half, lane);
+    // per-pair sums over rows of dW3, db2, db1, db3 and the squared residuals
+    {
+        const int i = (lane & 4) + ((lane >> 2) & 2) + (lane >> 4);
+        const int u = 8 * (4 * half + (i >> 1)) + 2 * t + (i & 1);
+        sm.red[pair][0][u] = sums_over_g(dw3, lane);
+        sm.red[pair][1][u] = sums_over_g(db2, lane);
+        sm.red[pair][2][u] = sums_over_g(db1, lane);
+    }
     sq = sum_over_g(sq);
     gsum = sum_over_g(gsum);
     if (lane == 0 && !half) {
         sm.red_s[pair][0] = gsum;
         sm.red_s[pair][1] = sq;
     }
-    __syncthreads();   // every warp's transposed tiles and partial sums
-    float* gW1 = ts.grad;
+    __syncthreads();   // every warp's tiles and partial sums
+    float* gW1 = sm.grad;
     float* gb1 = gW1 + kNF * kNH;
     float* gW2 = gb1 + kNH;
     float* gb2 = gW2 + kNH * kNH;
     float* gW3 = gb2 + kNH;
     // dW2 = bf(h1)^T bf(dz2) over the CTA's rows: 4 x 8 tiles of 16 x 8, four per
-    // warp, the two of each step sharing their rows of bf(h1)
-#pragma unroll 1
-    for (int tile = 2 * warp; tile < 32; tile += 16) {
-        const int u0 = 16 * (tile >> 3), v0 = 8 * (tile & 7);
-        float c[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    // warp (units u0 and u0 + 32, two v each); dW1 = bf(X)^T bf(dz1): 1 x 8 tiles
+    {
+        const int u0 = 16 * (warp >> 2), v0 = 16 * (warp & 3), w0 = 8 * warp;
+        float c[2][2][4] = {}, c1[4] = {};
 #pragma unroll
-        for (int kk = 0; kk < kTcRows / 16; ++kk) {
-            const int r = 16 * kk + 2 * t;
-            const uint32_t h[4] = {lds_u32(&sm.h1t[u0 + g][r]), lds_u32(&sm.h1t[u0 + g + 8][r]),
-                                   lds_u32(&sm.h1t[u0 + g][r + 8]), lds_u32(&sm.h1t[u0 + g + 8][r + 8])};
+        for (int kp = 0; kp < kTcRows / 32; ++kp) {
+            uint32_t b1[4];
+            ldsm4_t(b1, &sm.d1[32 * kp + lane][w0]);
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const uint32_t b[2] = {lds_u32(&sm.d2t[v0 + 8 * q + g][r]), lds_u32(&sm.d2t[v0 + 8 * q + g][r + 8])};
-                mma_bf16(c[q], h, b);
+            for (int h = 0; h < 2; ++h) {
+                const int r = 32 * kp + 16 * h;
+                uint32_t b[4], h0[4], h1[4], x[4];
+                ldsm4_t(b, &sm.d2[r + l15][v0 + l8]);
+                ldsm4_t(h0, &sm.h1[r + m15][u0 + m8]);
+                ldsm4_t(h1, &sm.h1[r + m15][u0 + 32 + m8]);
+                ldsm4_t(x, &sm.xb[r + m15][m8]);
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const uint32_t bq[2] = {b[2 * q], b[2 * q + 1]};
+                    mma_bf16(c[0][q], h0, bq);
+                    mma_bf16(c[1][q], h1, bq);
+                }
+                const uint32_t bq[2] = {b1[2 * h], b1[2 * h + 1]};
+                mma_bf16(c1, x, bq);
             }
         }
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int v = v0 + 8 * q + 2 * t;
-            *reinterpret_cast<float2*>(&gW2[(u0 + g) * kNH + v]) = make_float2(c[q][0], c[q][1]);
-            *reinterpret_cast<float2*>(&gW2[(u0 + g + 8) * kNH + v]) = make_float2(c[q][2], c[q][3]);
-        }
-    }
-    // dW1 = bf(X)^T bf(dz1): 1 x 8 tiles, one per warp
-    {
-        const int u0 = 8 * warp;
-        float c[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int kk = 0; kk < kTcRows / 16; ++kk) {
-            const int r = 16 * kk + 2 * t;
-            const uint32_t x[4] = {lds_u32(&sm.xt[g][r]), lds_u32(&sm.xt[g + 8][r]), lds_u32(&sm.xt[g][r + 8]),
-                                   lds_u32(&sm.xt[g + 8][r + 8])};
-            const uint32_t b[2] = {lds_u32(&sm.d1t[u0 + g][r]), lds_u32(&sm.d1t[u0 + g][r + 8])};
-            mma_bf16(c, x, b);
-        }
-        *reinterpret_cast<float2*>(&gW1[g * kNH + u0 + 2 * t]) = make_float2(c[0], c[1]);
-        *reinterpret_cast<float2*>(&gW1[(g + 8) * kNH + u0 + 2 * t]) = make_float2(c[2], c[3]);
+            for (int q = 0; q < 2; ++q) {
+                const int u = u0 + 32 * i + g, v = v0 + 8 * q + 2 * t;
+                *reinterpret_cast<float2*>(&gW2[u * kNH + v]) = make_float2(c[i][q][0], c[i][q][1]);
+                *reinterpret_cast<float2*>(&gW2[(u + 8) * kNH + v]) = make_float2(c[i][q][2], c[i][q][3]);
+            }
+        *reinterpret_cast<float2*>(&gW1[g * kNH + w0 + 2 * t]) = make_float2(c1[0], c1[1]);
+        *reinterpret_cast<float2*>(&gW1[(g + 8) * kNH + w0 + 2 * t]) = make_float2(c1[2], c1[3]);
     }
     // the row sums, added over the row groups in a fixed order
-    if (tid < kNH) {
-        float s3 = 0.f, sb2 = 0.f, sb1 = 0.f;
-        for (int w = 0; w < kTcWarps; ++w) {
-            s3 += sm.red[w][0][tid];
-            sb2 += sm.red[w][1][tid];
-            sb1 += sm.red[w][2][tid];
-        }
-        gW3[tid] = s3;
-        gb2[tid] = sb2;
-        gb1[tid] = sb1;
-    } else if (tid == kNH) {
+    if (tid < 3 * kNH) {
+        const int k = tid / kNH, u = tid % kNH;
+        float sum = 0.f;
+#pragma unroll
+        for (int w = 0; w < kTcWarps; ++w) sum += sm.red[w][k][u];
+        (k == 0 ? gW3 : k == 1 ? gb2 : gb1)[u] = sum;
+    } else if (tid == 3 * kNH) {
         float sg = 0.f, sl = 0.f;
         for (int w = 0; w < kTcWarps; ++w) {
             sg += sm.red_s[w][0];
             sl += sm.red_s[w][1];
         }
         gW3[kNH] = sg;                // db3
-        ts.loss = sl;
+        *loss = sl;
     }
 }
 
@@ -1042,18 +1110,21 @@ __global__ void __launch_bounds__(kTrainThreads) train_kernel(float* theta, floa
     extern __shared__ __align__(16) unsigned char tc_raw[];
     TrainSmem& sm = *reinterpret_cast<TrainSmem*>(tc_raw);
     cg::cluster_group cluster = cg::this_cluster();
-    const int ranks = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int rank = (int)cluster.block_rank();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int g = lane >> 2, t = lane & 3, pair = warp & 3;
-    const int share = (kNParams + ranks - 1) / ranks;
-    const int i0 = rank * share, n_own = max(0, min(share, kNParams - i0));
-    float *own_t = sm.own, *own_m = own_t + share, *own_v = own_m + share;
-    for (int i = tid; i < kNParams; i += kTrainThreads) tc_store_param(sm.tc, i, theta[i]);
-    for (int i = tid; i < n_own; i += kTrainThreads) {
-        own_t[i] = theta[i0 + i];
-        own_m[i] = am[i0 + i];
-        own_v[i] = av[i0 + i];
+    const int g = lane >> 2, t = lane & 3, pair = warp & 3, half = warp >> 2;
+    // this CTA's share of the parameters: pairs p0 .. p0 + n_own - 1
+    const int p0 = rank * kShare, n_own = min(kShare, kPairs - p0);
+    const int parts = (batch + kTcRows - 1) / kTcRows;   // CTAs with rows
+    auto pair_of = [](const float* p, int i) { return make_float2(p[i], i + 1 < kNParams ? p[i + 1] : 0.f); };
+    for (int p = tid; p < kPairs; p += kTrainThreads) store_operands(operand_pair(sm, 2 * p), pair_of(theta, 2 * p));
+    for (int p = tid; p < n_own; p += kTrainThreads) {
+        sm.own_t[p] = pair_of(theta, 2 * (p0 + p));
+        sm.own_m[p] = pair_of(am, 2 * (p0 + p));
+        sm.own_v[p] = pair_of(av, 2 * (p0 + p));
     }
+    if (tid < 3) sm.grad[kNParams + tid] = 0.f;
+    float* loss_slot = cluster.map_shared_rank(sm.loss, 0) + rank;
     const int my_row = rank * kTcRows + tid;   // of the mini-batch
     auto request = [&](int step, int slot) {
         if (tid < kTcRows && my_row < batch) {
@@ -1066,59 +1137,102 @@ __global__ void __launch_bounds__(kTrainThreads) train_kernel(float* theta, floa
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     request(0, 0);
+    cluster_arrive();   // every CTA runs: its shared memory may be written
+    cluster_wait();
     const float scale = 1.0f / (float)batch;
+    float c1, c2;   // Adam's, of the step
+    auto corrections = [&](int step) {
+        c1 = 1.f - powf(0.9f, (float)(adam0 + 1 + step));
+        c2 = 1.f - powf(0.999f, (float)(adam0 + 1 + step));
+    };
+    corrections(0);
     for (int k = 0; k < steps; ++k) {
         const int slot = k & 1;
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();   // the rows of this step, from every thread
-        uint32_t ax[2][4];
-        float y[2][2];
-        bool act[2][2];
+        if (rank < parts) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();   // the rows of this step, from every thread
+            uint32_t ax[2][4];
+            float y[2][2];
+            bool act[2][2];
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
+            for (int mt = 0; mt < 2; ++mt) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int r = pair * 32 + 16 * mt + g + 8 * h;
-                act[mt][h] = rank * kTcRows + r < batch;
-                float2 lo = make_float2(0.f, 0.f), hi = make_float2(0.f, 0.f);
-                y[mt][h] = 0.f;
-                if (act[mt][h]) {
-                    lo = *reinterpret_cast<const float2*>(&sm.x[slot][r][2 * t]);
-                    hi = *reinterpret_cast<const float2*>(&sm.x[slot][r][2 * t + 8]);
-                    y[mt][h] = sm.y[slot][r];
+                for (int h = 0; h < 2; ++h) {
+                    const int r = pair * 32 + 16 * mt + g + 8 * h;
+                    act[mt][h] = rank * kTcRows + r < batch;
+                    float2 lo = make_float2(0.f, 0.f), hi = make_float2(0.f, 0.f);
+                    y[mt][h] = 0.f;
+                    if (act[mt][h]) {
+                        lo = *reinterpret_cast<const float2*>(&sm.x[slot][r][2 * t]);
+                        hi = *reinterpret_cast<const float2*>(&sm.x[slot][r][2 * t + 8]);
+                        y[mt][h] = sm.y[slot][r];
+                    }
+                    ax[mt][h] = pack_bf16(lo.x, lo.y);        // A regs 0 (row g) and 1 (row g + 8)
+                    ax[mt][2 + h] = pack_bf16(hi.x, hi.y);    // A regs 2 and 3
+                    if (half == mt) {
+                        *reinterpret_cast<uint32_t*>(&sm.xb[r][2 * t]) = ax[mt][h];
+                        *reinterpret_cast<uint32_t*>(&sm.xb[r][2 * t + 8]) = ax[mt][2 + h];
+                    }
                 }
-                tc_row(sm.tc, ax, mt, h, lo, hi, pair, g, t);   // (both halves write the same)
             }
+            train_gradient(sm, ax, act, y, scale, loss_slot, tid);
         }
+        cluster_arrive();   // every CTA's gradient
         if (k + 1 < steps) request(k + 1, slot ^ 1);
-        train_gradient(sm, ax, act, y, scale, tid);
-        cluster.sync();   // every CTA's gradient
-        const float c1 = 1.f - powf(0.9f, (float)(adam0 + 1 + k)), c2 = 1.f - powf(0.999f, (float)(adam0 + 1 + k));
-        for (int i = tid; i < n_own; i += kTrainThreads) {
-            // the eight requests leave together (one after the other they were
-            // half of a step's time); absent CTAs repeat this one's
-            float part[kMaxTrainCtas];
+        cluster_wait();
+        // the requests of both of a thread's pairs leave together (one after the
+        // other they were half of a step's time)
+        constexpr int kOwn = (kShare + kTrainThreads - 1) / kTrainThreads;
+        float2 part[kOwn][kTrainCtas];
 #pragma unroll
-            for (int b = 0; b < kMaxTrainCtas; ++b)
-                part[b] = cluster.map_shared_rank(sm.grad, b < ranks ? b : rank)[i0 + i];
-            float gr = 0.f;
+        for (int i = 0; i < kOwn; ++i) {
+            const int p = tid + i * kTrainThreads;
+            float* mine = sm.grad + 2 * (p0 + p);
 #pragma unroll
-            for (int b = 0; b < kMaxTrainCtas; ++b)
-                if (b < ranks) gr += part[b];
-            adam_update(gr, c1, c2, lr, own_m[i], own_v[i], own_t[i]);
-            for (int b = 0; b < ranks; ++b) tc_store_param(*cluster.map_shared_rank(&sm.tc, b), i0 + i, own_t[i]);
+            for (int b = 0; b < kTrainCtas; ++b)
+                if (p < n_own && b < parts)
+                    part[i][b] = *reinterpret_cast<const float2*>(cluster.map_shared_rank(mine, b));
         }
-        if (rank == 0 && tid == 0) {
+#pragma unroll
+        for (int i = 0; i < kOwn; ++i) {
+            const int p = tid + i * kTrainThreads;
+            if (p >= n_own) break;
+            float2 gr = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int b = 0; b < kTrainCtas; ++b)
+                if (b < parts) {
+                    gr.x += part[i][b].x;
+                    gr.y += part[i][b].y;
+                }
+            float2 m = sm.own_m[p], v = sm.own_v[p], th = sm.own_t[p];
+            adam_update(gr.x, c1, c2, lr, m.x, v.x, th.x);
+            adam_update(gr.y, c1, c2, lr, m.y, v.y, th.y);
+            sm.own_m[p] = m;
+            sm.own_v[p] = v;
+            sm.own_t[p] = th;
+            const OperandPair at = operand_pair(sm, 2 * (p0 + p));
+#pragma unroll
+            for (int b = 0; b < kTrainCtas; ++b) store_operands({cluster.map_shared_rank(at.at, b), at.half}, th);
+        }
+        if (rank == 0 && tid == kTrainThreads - 1) {
             float tot = 0.f;
-            for (int b = 0; b < ranks; ++b) tot += *cluster.map_shared_rank(&sm.loss, b);
+            for (int b = 0; b < parts; ++b) tot += sm.loss[b];
             loss[k] = tot;
         }
-        cluster.sync();   // every CTA's operands; the gradients are read
+        cluster_arrive();   // every CTA's operands; the gradients are read
+        corrections(k + 1);
+        cluster_wait();
     }
-    for (int i = tid; i < n_own; i += kTrainThreads) {
-        theta[i0 + i] = own_t[i];
-        am[i0 + i] = own_m[i];
-        av[i0 + i] = own_v[i];
+    for (int p = tid; p < n_own; p += kTrainThreads) {
+        const int i = 2 * (p0 + p);
+        theta[i] = sm.own_t[p].x;
+        am[i] = sm.own_m[p].x;
+        av[i] = sm.own_v[p].x;
+        if (i + 1 < kNParams) {
+            theta[i + 1] = sm.own_t[p].y;
+            am[i + 1] = sm.own_m[p].y;
+            av[i + 1] = sm.own_v[p].y;
+        }
     }
 }
 
@@ -1221,32 +1335,23 @@ cudaError_t surrogate_step(const float* theta_in, const float* X, const float* y
     return cudaGetLastError();
 }
 
-namespace {
-
-size_t train_smem(int ranks) {
-    return sizeof(TrainSmem) + 3 * size_t((kNParams + ranks - 1) / ranks) * sizeof(float);
-}
-
-}  // namespace
-
-bool surrogate_train_fits(int batch) { return batch <= kMaxTrainCtas * kTcRows; }
+bool surrogate_train_fits(int batch) { return batch <= kTrainCtas * kTcRows; }
 
 cudaError_t surrogate_train_steps(float* theta, float* m, float* v, const float* X, const float* y, int count,
                                   int batch, int steps, int adam_t, float lr, uint32_t k0, uint32_t k1, float* loss,
                                   cudaStream_t s) {
-    const int ranks = (batch + kTcRows - 1) / kTcRows;
-    if (ranks < 1 || ranks > kMaxTrainCtas) return cudaErrorInvalidValue;
-    const size_t smem = train_smem(ranks);
+    if (batch < 1 || !surrogate_train_fits(batch)) return cudaErrorInvalidValue;
+    const size_t smem = sizeof(TrainSmem);
     cudaError_t err = cudaFuncSetAttribute(train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(ranks);
+    cfg.gridDim = dim3(kTrainCtas);
     cfg.blockDim = dim3(kTrainThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = ranks;
+    at.val.clusterDim.x = kTrainCtas;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
