@@ -62,13 +62,14 @@ __device__ __forceinline__ float r2_exact(const Geometry& g, float qx, float qy,
 __device__ float features_all(const SweepParams& P, int w, int N, float qx, float qy, float qz, int skip,
                               float (&F)[kNF], int lane) {
     const float4* pos = P.pos + size_t(w) * P.nmax;
+    const float inv_rc = 1.0f / P.g.rc;
     float e = 0.f;
     for (int j = lane; j < N; j += 32) {
         if (j == skip) continue;
         const PairTab& t = j < P.n_cluster ? P.gAB : P.gg;
         const float r2 = r2_exact(P.g, qx, qy, qz, pos[j]);
         if (r2 < P.g.rc2) {
-            add_features(F, r2, t.eps, P.g.rc);
+            add_features(F, r2, t.eps, P.g.rc, inv_rc);
             e += phi_of_r2(r2, t);
         }
     }
@@ -77,7 +78,7 @@ __device__ float features_all(const SweepParams& P, int w, int N, float qx, floa
         const PairTab& t = surf_tab(P, (int)at.w);
         const float r2 = r2_exact(P.g, qx, qy, qz, at);
         if (r2 < P.g.rc2) {
-            add_features(F, r2, t.eps, P.g.rc);
+            add_features(F, r2, t.eps, P.g.rc, inv_rc);
             e += phi_of_r2(r2, t);
         }
     }
