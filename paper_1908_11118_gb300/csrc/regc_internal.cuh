@@ -277,9 +277,9 @@ __device__ __forceinline__ float pair_phi(float dx, float dy, float dz, float rc
 // final subtraction rounds.
 __device__ __forceinline__ float min_image_exact(float q, float p, float L, float hL) {
     const float e = __fsub_rn(q, p);
-    if (e > hL) return __fsub_rn(__fsub_rn(q, L), p);
-    if (e < -hL) return __fsub_rn(q, __fsub_rn(p, L));
-    return e;
+    const float qs = e > hL ? __fsub_rn(q, L) : q;
+    const float ps = e < -hL ? __fsub_rn(p, L) : p;
+    return __fsub_rn(qs, ps);
 }
 
 __device__ __forceinline__ const PairTab& surf_tab(const SweepParams& P, int type) {
