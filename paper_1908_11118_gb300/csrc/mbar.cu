@@ -731,7 +731,9 @@ __global__ void __launch_bounds__(256) sp_screen_kernel(const __grid_constant__ 
 // warp-wide FP64 instruction costs the narrow FP64 pipe the same whatever its
 // active lanes, and the row is written in whole sectors.  (One thread per bin
 // scanning every state took 3.5 times as long on 1024 states: each warp paid
-// for the union of its 32 bins' states and wrote 32 separate rows.)
+// for the union of its 32 bins' states and wrote 32 separate rows.)  What bounds
+// it is FP64; t_sb is therefore kept in the row between the two passes: 114
+// million entries 6.16 -> 5.5 ms.
 constexpr int kRowWarps = 8;
 template <bool TWO>
 __global__ void __launch_bounds__(32 * kRowWarps) sp_rows_kernel(const __grid_constant__ MbarDev m, SpDev p) {
@@ -748,15 +750,17 @@ __global__ void __launch_bounds__(32 * kRowWarps) sp_rows_kernel(const __grid_co
         for (uint32_t bits = p.mask[at]; bits; bits &= bits - 1u) ci[o++] = 32 * w + __ffs(bits) - 1;
     }
     __syncwarp();
-    auto term = [&](int e) {
-        const int s = ci[e];
-        return p.gs[s] - u_of<TWO>(m.a[s], m.c[s], TWO ? m.c2[s] : 0.0, E, N, N2);
-    };
+    double* cv = p.cv + r0;
     double M = -INFINITY;
-    for (int e = lane; e < n; e += 32) M = fmax(M, term(e));
+    for (int e = lane; e < n; e += 32) {
+        const int s = ci[e];
+        const double t = p.gs[s] - u_of<TWO>(m.a[s], m.c[s], TWO ? m.c2[s] : 0.0, E, N, N2);
+        cv[e] = t;   // (read back by this lane: cheaper than taking it again in FP64)
+        M = fmax(M, t);
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
-    for (int e = lane; e < n; e += 32) p.cv[r0 + e] = exp(term(e) - M);
+    for (int e = lane; e < n; e += 32) cv[e] = exp(cv[e] - M);
     if (lane == 0) {
         p.M[b] = M;
         p.H[b] = exp(m.lnH[b]);
@@ -835,9 +839,8 @@ __global__ void __launch_bounds__(kDThreads) sp_d_kernel(const __grid_constant__
         __syncthreads();
     }
     if (!FINAL && blockIdx.x == 0 && threadIdx.x == 0) p.t_out[0] = global_ns();
-    const long long gt = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long b = gt / kDLanes;
-    const int sub = (int)(gt % kDLanes);
+    const int lane = threadIdx.x & 31, sub = lane % kDLanes;
+    const long long b = ((long long)blockIdx.x * kDThreads + threadIdx.x) / kDLanes;
     const bool act = b < m.B;
     double d0 = 0.0, d1 = 0.0;
     if (act) {
@@ -898,19 +901,42 @@ __global__ void __launch_bounds__(kDThreads) sp_d_kernel(const __grid_constant__
 // and to the host's page-locked buffer; an empty sum is reported.  The last
 // state of all writes the map's number seq there too, which the host waits for
 // (it sees it microseconds before the stream's own completion).
+//
+// What bounds it: memory, 12 bytes an entry, as long as enough requests are on
+// the way.  A thread requests its next four entries before it gathers V for
+// these: 114 million entries (507759 bins, 1024 states) 368 -> 243 us, against
+// 202 for the 1.37 GB; 14 million 60 -> 48.
 constexpr long long kPiece = 32768;
 __global__ void __launch_bounds__(kFThreads) sp_fp_kernel(const __grid_constant__ MbarDev m,
                                                           const __grid_constant__ SpDev p, unsigned seq) {
     const long long e0 = p.pc_begin[blockIdx.x], e1 = p.pc_begin[blockIdx.x + 1];
     double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
     long long e = e0 + threadIdx.x;
-    for (; e + 3 * kFThreads < e1; e += 4 * kFThreads) {
-        const int b0 = p.bi[e], b1 = p.bi[e + kFThreads], b2 = p.bi[e + 2 * kFThreads], b3 = p.bi[e + 3 * kFThreads];
-        const double k0 = p.bv[e], k1 = p.bv[e + kFThreads], k2 = p.bv[e + 2 * kFThreads], k3 = p.bv[e + 3 * kFThreads];
-        a0 = fma(k0, p.V[b0], a0);
-        a1 = fma(k1, p.V[b1], a1);
-        a2 = fma(k2, p.V[b2], a2);
-        a3 = fma(k3, p.V[b3], a3);
+    int b[4];
+    double k[4];
+    auto request = [&](long long at) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            b[q] = p.bi[at + q * kFThreads];
+            k[q] = p.bv[at + q * kFThreads];
+        }
+    };
+    bool full = e + 3 * kFThreads < e1;
+    if (full) request(e);
+    while (full) {
+        double v[4], kk[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            v[q] = __ldg(p.V + b[q]);
+            kk[q] = k[q];
+        }
+        e += 4 * kFThreads;
+        full = e + 3 * kFThreads < e1;
+        if (full) request(e);   // the next four are under way while these are added
+        a0 = fma(kk[0], v[0], a0);
+        a1 = fma(kk[1], v[1], a1);
+        a2 = fma(kk[2], v[2], a2);
+        a3 = fma(kk[3], v[3], a3);
     }
     for (; e < e1; e += kFThreads) a0 = fma(p.bv[e], p.V[p.bi[e]], a0);
     const double acc = block_sum((a0 + a1) + (a2 + a3));
