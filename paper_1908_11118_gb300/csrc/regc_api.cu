@@ -205,10 +205,10 @@ regc_status init_grid(const regc_potential* pot, const regc_surface* surf, const
     // A round of K costs one evaluation and K commits in order, so it pays
     // while the issue slots are idle.  Microseconds of a ten-sweep launch with
     // 1 / 2 / 4 warps (SMs: 152):
-    //   fcc(111):  64 walkers 310 / 273 / 236, 256: 316 / 272 / 250,
-    //              512: 314 / 286 / 264, 1024: 338 / 333 / 463
-    //   A18:       160: 136 / 111 / 89, 640: 181 / 172 / 200
-    //   fcc(100):  256: 210 / 196 / 191, 4096: 458 / 784 / 1083
+    //   fcc(111):  64 walkers 265 / 240 / 217, 256: 268 / 241 / 231,
+    //              512: 268 / 254 / 242, 1024: 285 / 452 / 429
+    //   A18:       160: 108 / 91 / 75, 640: 140 / 138 / 168
+    //   fcc(100):  256: 170 / 174 / 171, 4096: 334 / 702 / 962
     // REGC_WARPS_PER_WALKER overrides the choice.
     int W = 1, sms = 0;
     {
