@@ -37,10 +37,10 @@
 // through shared memory and the draws made one move at a time; it took 572 at
 // 4.9 (ncu: 1.9 of them waiting for a fixed latency, 1.0 for shared memory or a
 // shuffle, 0.4 for a branch, 0.3 for the instruction fetch) without them, and
-// fewer since the geometry is compiled in (make_hot) and cells out of reach are
+// 513 at 4.8 with the geometry compiled in (make_hot) and cells out of reach
 // left out (stencil_list).  Steps of ten sweeps, before / after all of it: 16
-// fcc(100) replicas 406 / 192 us with the walkers read back, a hundred REGC steps
-// of 160 A18 replicas 2.2 / 0.88 ms, 4096 clusters 950 / 456 us, the 1024-replica
+// fcc(100) replicas 406 / 184 us with the walkers read back, a hundred REGC steps
+// of 160 A18 replicas 2.2 / 0.85 ms, 4096 clusters 950 / 456 us, the 1024-replica
 // grid 400 / 322 us.  With delayed acceptance the code of the features stands
 // once instead of six times and the kernel is no longer bound by the instruction
 // fetch: 1930 / 760 us.

@@ -49,3 +49,30 @@ def test_cluster_training_shapes(batch):
     lb, tb = trained(3, 4)
     assert np.array_equal(la, lb) and np.array_equal(ta, tb)
     assert np.isfinite(ta).all() and not np.array_equal(ta, t1)
+
+
+@pytest.mark.parametrize("layer", [0, 1, 2])
+def test_cluster_training_far_units(layer):
+    """Units far below zero (x < -80, and where exp(-x) overflows), whose SiLU
+    derivatives take the general form: in layer 1, layer 2 or both, next to
+    ordinary units.  The same comparison as above."""
+    p = W.fcc100_small(L=2, M=2, seed=9)
+    rng = np.random.default_rng(layer)
+    X = rng.gamma(1.0, 0.5, (300, 16)).astype(np.float32)
+    y = (X @ rng.normal(size=16) - 1.0).astype(np.float32)
+    th = SG.init_params(3, scale=1.0).astype(np.float32)
+    for on, b in ((layer != 1, 1024), (layer != 0, 1024 + 64 + 4096)):   # b1, b2
+        if on:
+            th[b:b + 64:4] = -84.0
+            th[b + 1:b + 64:4] = -200.0
+    key = (int(p.seed) & 0xFFFFFFFF, int(p.seed) >> 32)
+    rows = SG.batch_rows(1, 200, len(y), key)
+    loss, grad = surrogate_gradient(th, X[rows], y[rows], tensor_cores=True)
+    g = Regc(p)
+    g.surrogate_set(th)
+    g.surrogate_set_dataset(X, y, capacity=512)
+    l1, t1 = g.surrogate_train(1, 200, 1e-3), g.surrogate_get()
+    assert abs(l1[0] - loss) <= 1e-6 * abs(loss)
+    step = -1e-3 * grad.astype(np.float64) / (np.abs(grad.astype(np.float64)) + 1e-8)
+    assert np.all(np.abs(t1 - (th + step)) <= 2e-5 * 1e-3 + 2.0 ** -23 * np.abs(th))
+    assert np.isfinite(t1).all()
