@@ -594,9 +594,10 @@ __global__ void prep_bins_kernel(int B, const double* H, double* lnH) {
 // matrix holds to e^-50 while the spread of the drift, max_s (f_s - f_ref,s)
 // - min_s (f_s - f_ref,s), is at most kSpreadAcc: a dropped entry then weighs
 // at most e^(-kKeep + kSpreadAcc) = e^-50 of the largest term of its bin (a
-// uniform shift of f changes nothing), so the (at most 65536) dropped terms
-// of d_b stay below 1e-17 of it, and those of a state's sum below 1e-17 of
-// it too while its observations Omega_s are not below N_obs / S e^-13.  Far
+// uniform shift of f changes nothing), so the at most S dropped terms of d_b
+// stay below S e^-50 of it (1.3e-17 for the 65536 states a handle can have),
+// and those of a state's sum too while its observations Omega_s are not below
+// N_obs / S e^-13.  Far
 // from the fixed point the iteration runs on the matrix until the spread
 // exceeds kSpreadMax (its map then errs by at most e^-10 relative, which
 // changes the path, not the end point); convergence is accepted only on a
@@ -620,7 +621,7 @@ struct SpDev {
     int* ci;         // [nnz] their states, ascending within a bin
     double* cv;      // [nnz] K_sb
     uint32_t* mask;  // [words][B] kept states 32 w .. 32 w + 31 of bin b
-    uint16_t* pref;  // [words][B] kept states of bin b before word w
+    uint32_t* pref;  // [words][B] kept states of bin b before word w (any number: S has no upper bound)
     int words;       // ceil(S / 32)
     int chunk;       // bins per chunk of the by-state order, a multiple of 32
     int n_chunk;
@@ -717,7 +718,7 @@ __global__ void __launch_bounds__(256) sp_screen_kernel(const __grid_constant__ 
                                      ? 1u : 0u) << q;
                     const size_t at = size_t((k0 + q0) >> 5) * m.B + b;
                     p.mask[at] = bits;
-                    p.pref[at] = (uint16_t)cnt;
+                    p.pref[at] = (uint32_t)cnt;
                     cnt += __popc(bits);
                 }
             }
@@ -746,7 +747,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) sp_rows_kernel(const __grid_co
     int* ci = p.ci + r0;
     for (int w = lane; w < p.words; w += 32) {
         const size_t at = size_t(w) * m.B + b;
-        int o = p.pref[at];
+        int o = (int)p.pref[at];
         for (uint32_t bits = p.mask[at]; bits; bits &= bits - 1u) ci[o++] = 32 * w + __ffs(bits) - 1;
     }
     __syncwarp();
@@ -1149,7 +1150,7 @@ struct SparseMat {
         const size_t SC = S * p.n_chunk, words = size_t(p.words) * B;
         const size_t nt = std::max((B + kScanChunk - 1) / kScanChunk, (SC + kScanChunk - 1) / kScanChunk) + 1;
         const size_t n8 = (B + 1) + (SC + 1) + 3 * B + 3 * S + nt;
-        cudaError_t e = cudaMallocAsync(&fixed, n8 * 8 + words * 6 + (S + 1) * 4 + 16, s);
+        cudaError_t e = cudaMallocAsync(&fixed, n8 * 8 + words * 8 + (S + 1) * 4, s);
         if (e != cudaSuccess) {
             fixed = nullptr;
             return e;
@@ -1166,9 +1167,9 @@ struct SparseMat {
         p.w = p.gs + S;
         tmp = reinterpret_cast<long long*>(p.w + S);
         p.mask = reinterpret_cast<uint32_t*>(tmp + nt);
-        p.done = reinterpret_cast<int*>(p.mask + words);
+        p.pref = p.mask + words;
+        p.done = reinterpret_cast<int*>(p.pref + words);
         p.all_done = p.done + S;
-        p.pref = reinterpret_cast<uint16_t*>(p.all_done + 1);
         e = cudaMemsetAsync(p.rp, 0, sizeof(long long), s);
         if (e == cudaSuccess) e = cudaMemsetAsync(p.cp, 0, sizeof(long long), s);
         return e;

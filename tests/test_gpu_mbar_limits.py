@@ -1,0 +1,39 @@
+"""The sparse kernel matrix at the limits of its indices, of the memory it may
+take and of its waits."""
+import numpy as np
+import pytest
+
+from oracle import mbar as OM
+from paper_1908_11118_gb300 import build as B
+from paper_1908_11118_gb300 import mbar_last_info, mbar_solve
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    B.build()
+
+
+def close_states(S, bins, seed):
+    """S states so close in (kT, mu) that every bin keeps the terms of all of them."""
+    rng = np.random.default_rng(seed)
+    kT, mu = np.linspace(1.0, 1.05, S), np.linspace(-3.5, -3.4, S)
+    N = np.sort(rng.integers(0, 25, bins))
+    E = -2.0 * N + rng.normal(size=bins) * (0.5 + 0.3 * np.sqrt(N))
+    H = rng.uniform(1.0, 50.0, bins)
+    return kT, mu, np.full(S, H.sum() / S), N, E, H
+
+
+@pytest.mark.parametrize("S", [65536, 65537, 65600])
+def test_rows_of_more_than_65535_states(S):
+    """The number of a row's entries before a word of 32 states passes 65535."""
+    kT, mu, omega, N, E, H = close_states(S, 40, seed=S)
+    f, D, _ = mbar_solve(kT, mu, 1.0, omega, N, E, H, tol=1e-11)
+    info = mbar_last_info()
+    assert info["path"] == 1 and info["lse_maps"] == 0 and info["nnz"] == S * len(N)
+    # one FP64 map of the oracle from f stays there (the convergence asked for,
+    # 1e-11, and the rounding of sums of up to 7e4 terms of size e^+-100)
+    f1, D1, _, _ = OM.solve(kT, mu, 1.0, omega, N, E, H, max_iter=1, f0=f)
+    np.testing.assert_allclose(f, f1, atol=1e-9)
+    np.testing.assert_allclose(D, D1, atol=1e-9)
