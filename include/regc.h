@@ -613,10 +613,11 @@ REGC_API regc_status regc_structure_timing(regc_handle *h, double *ms_mbar, doub
  * D_b = ln sum_k omega_k exp(f_k - u_k(b)).  Runs on cuda_stream.
  * Device memory: besides O(S + B) buffers, when every omega_k > 0 the
  * iterations use the kept entries of the kernel matrix (those within e^-70
- * of the largest of their bin, stored by bin and by state: 24 bytes each),
- * allocated on the stream for the duration of the call when they fit in half
- * the free device memory (otherwise they run without it; the result is the
- * same fixed point).  regc_reweight, regc_reweight2 and
+ * of the largest of their bin, stored by bin and by state: 24 bytes each) and
+ * a bit mask of them with its row sums (8 bytes per bin and 32 states),
+ * allocated on the stream for the duration of the call when together they fit
+ * in half the free device memory (otherwise they run without it; the result is
+ * the same fixed point).  regc_reweight, regc_reweight2 and
  * regc_structure_reweight solve the same way; regc_mbar_last_info reports
  * what the last solve did. */
 REGC_API regc_status regc_mbar_solve(int S, const double *kT, const double *mu, double lambda0,

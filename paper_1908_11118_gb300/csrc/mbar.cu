@@ -1120,6 +1120,7 @@ struct SparseMat {
     void* entries = nullptr;   // cap entries: cv, bv (double), ci, bi (int)
     void* pieces = nullptr;    // pc_begin, pc_sum, pc_state, pc_first for up to pc_cap pieces
     long long cap = 0, nnz = 0, pc_cap = 0, n_pieces = 0;
+    size_t budget = 0;         // bytes left for the entries: half the memory free at the start less `fixed`
     int sms = 152;
     std::vector<long long> h_begin;   // pc_begin and pc_state, pc_first as last uploaded
     std::vector<int> h_index;
@@ -1132,6 +1133,8 @@ struct SparseMat {
         if (fixed) cudaFreeAsync(fixed, s);
     }
 
+    // cudaErrorMemoryAllocation where the masks alone pass half the free device
+    // memory (nothing is allocated then).
     cudaError_t init(const MbarDev& m) {
         const size_t B = size_t(m.B), S = size_t(m.S);
         int dev = 0;
@@ -1150,7 +1153,13 @@ struct SparseMat {
         const size_t SC = S * p.n_chunk, words = size_t(p.words) * B;
         const size_t nt = std::max((B + kScanChunk - 1) / kScanChunk, (SC + kScanChunk - 1) / kScanChunk) + 1;
         const size_t n8 = (B + 1) + (SC + 1) + 3 * B + 3 * S + nt;
-        cudaError_t e = cudaMallocAsync(&fixed, n8 * 8 + words * 8 + (S + 1) * 4, s);
+        const size_t bytes = n8 * 8 + words * 8 + (S + 1) * 4;
+        size_t fr = 0, tot = 0;
+        cudaError_t e = cudaMemGetInfo(&fr, &tot);
+        if (e != cudaSuccess) return e;
+        if (bytes > fr / 2) return cudaErrorMemoryAllocation;
+        budget = fr / 2 - bytes;
+        e = cudaMallocAsync(&fixed, bytes, s);
         if (e != cudaSuccess) {
             fixed = nullptr;
             return e;
@@ -1175,8 +1184,9 @@ struct SparseMat {
         return e;
     }
 
-    // *ok is false when the entries do not fit (half the free device memory)
-    // or the two orders disagree; the caller then iterates on log-sum-exps.
+    // *ok is false when the entries do not fit (with the masks, half the device
+    // memory free at the start) or the two orders disagree; the caller then
+    // iterates on log-sum-exps.
     template <bool TWO>
     cudaError_t build(const MbarDev& m, bool* ok) {
         *ok = false;
@@ -1208,7 +1218,7 @@ struct SparseMat {
             e = cudaMemGetInfo(&fr, &tot);
             if (e != cudaSuccess) return e;
             const size_t need = size_t(n_h) * 24;
-            if (need > fr / 2) return cudaSuccess;
+            if (need > fr / 2 || need > budget) return cudaSuccess;
             if (cudaMallocAsync(&entries, need, s) != cudaSuccess) {
                 entries = nullptr;
                 (void)cudaGetLastError();   // out of memory is not sticky

@@ -58,8 +58,9 @@ MbarInfo mbar_last_info();
 // With allow_matrix (and every state sampled) the iterations run on the
 // kept entries of the kernel matrix K_sb = exp(-u_s(b) + ln Omega_s + f_ref,s
 // - max_k(...)) (those within e^-70 of their bin's largest), allocated on the
-// stream for the duration of the call when they fit in half the free device
-// memory; otherwise on log-sum-exps of the energies.
+// stream for the duration of the call when they fit, with the mask they are
+// built from, in half the free device memory; otherwise on log-sum-exps of the
+// energies.
 // x0 (host, S values, optional) is the starting point instead of f = 0.
 cudaError_t mbar_solve_dev(const MbarDev& m, double tol, int max_iter, int* iters_out,
                            cudaStream_t s, bool allow_matrix = true, const double* x0 = nullptr);

@@ -1,5 +1,7 @@
 """The sparse kernel matrix at the limits of its indices, of the memory it may
 take and of its waits."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -37,3 +39,42 @@ def test_rows_of_more_than_65535_states(S):
     f1, D1, _, _ = OM.solve(kT, mu, 1.0, omega, N, E, H, max_iter=1, f0=f)
     np.testing.assert_allclose(f, f1, atol=1e-9)
     np.testing.assert_allclose(D, D1, atol=1e-9)
+
+
+class Pool:
+    """The most that the device's default memory pool held at once since reset()."""
+    USED_MEM_HIGH = 8
+
+    def __init__(self):
+        self.cu = ctypes.CDLL("libcuda.so.1")
+        dev, self.pool = ctypes.c_int(), ctypes.c_void_p()
+        assert self.cu.cuDeviceGet(ctypes.byref(dev), 0) == 0
+        assert self.cu.cuDeviceGetDefaultMemPool(ctypes.byref(self.pool), dev) == 0
+
+    def reset(self):
+        assert self.cu.cuMemPoolSetAttribute(self.pool, self.USED_MEM_HIGH, ctypes.byref(ctypes.c_uint64(0))) == 0
+
+    def high(self):
+        v = ctypes.c_uint64()
+        assert self.cu.cuMemPoolGetAttribute(self.pool, self.USED_MEM_HIGH, ctypes.byref(v)) == 0
+        return v.value
+
+
+def test_masks_count_against_half_the_free_memory():
+    """1.2e6 bins of 4096 states take 0.9 GB or more of masks: with 1.6 GB free the
+    solve does without the matrix and never holds half of what is free."""
+    torch = pytest.importorskip("torch")
+    left = 1_600_000_000
+    torch.cuda.init()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - left, dtype=torch.uint8, device="cuda")
+    try:
+        kT, mu, omega, N, E, H = close_states(4096, 1_200_000, seed=1)
+        pool = Pool()
+        torch.cuda.synchronize()
+        pool.reset()
+        mbar_solve(kT, mu, 1.0, omega, N, E, H, max_iter=1)
+        assert pool.high() < left // 2
+        assert mbar_last_info()["path"] == 0
+    finally:
+        del hold
+        torch.cuda.empty_cache()
