@@ -617,7 +617,9 @@ REGC_API regc_status regc_structure_timing(regc_handle *h, double *ms_mbar, doub
  * a bit mask of them with its row sums (8 bytes per bin and 32 states),
  * allocated on the stream for the duration of the call when together they fit
  * in half the free device memory (otherwise they run without it; the result is
- * the same fixed point).  regc_reweight, regc_reweight2 and
+ * the same fixed point).  The host waits after every map: it spins, unless the
+ * device's scheduling flags ask for yielding or blocking waits, which it then
+ * follows.  regc_reweight, regc_reweight2 and
  * regc_structure_reweight solve the same way; regc_mbar_last_info reports
  * what the last solve did. */
 REGC_API regc_status regc_mbar_solve(int S, const double *kT, const double *mu, double lambda0,
@@ -632,8 +634,9 @@ REGC_API regc_status regc_mbar_solve(int S, const double *kT, const double *mu, 
  * self-consistent equations), matrix builds, maps taken on log-sum-exps (no
  * matrix, or a state without a kept entry far from the fixed point), the kept
  * entries of the last build, its S and B, the device milliseconds of the
- * matrix builds and of the maps on the matrix (CUDA events on the solve's
- * stream), and the number of those maps.  regc_reweight and regc_reweight2
+ * matrix builds (CUDA events on the solve's stream) and of the maps on the
+ * matrix (the device's global timer, read by the first and the last kernel of
+ * a map), and the number of those maps.  regc_reweight and regc_reweight2
  * start a problem of at least 65536 bins from the solution of the same
  * problem with 16 energy bins merged into one (solved to 1e-6; same fixed
  * point, fewer matrix builds): coarse_iterations, coarse_B, coarse_builds

@@ -1291,7 +1291,12 @@ struct HostBlock {
     unsigned long long* t = nullptr;
     int* empty = nullptr;
     volatile unsigned* seq = nullptr;
+    bool spin = true;   // the process's scheduling flags let a waiting thread keep its core
     bool init(int S) {
+        unsigned flags = 0;
+        if (cudaGetDeviceFlags(&flags) != cudaSuccess) (void)cudaGetLastError();
+        flags &= cudaDeviceScheduleMask;
+        spin = flags != cudaDeviceScheduleYield && flags != cudaDeviceScheduleBlockingSync;
         if (cudaHostAlloc(&block, size_t(2 * S + 4) * sizeof(double), cudaHostAllocDefault) != cudaSuccess) {
             block = nullptr;
             (void)cudaGetLastError();
@@ -1306,8 +1311,10 @@ struct HostBlock {
         return true;
     }
     // Wait for map number n: until its number arrives, or the stream has ended
-    // or failed (asked now and then).
+    // or failed (asked now and then).  Where the process asked for waits that
+    // give up the core, by the stream's own synchronisation.
     cudaError_t wait(unsigned n, cudaStream_t s) const {
+        if (!spin) return cudaStreamSynchronize(s);
         for (unsigned spin = 1; *seq != n; ++spin) {
             if ((spin & 4095u) != 0u) continue;
             const cudaError_t e = cudaStreamQuery(s);
