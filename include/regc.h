@@ -619,7 +619,9 @@ REGC_API regc_status regc_structure_timing(regc_handle *h, double *ms_mbar, doub
  * in half the free device memory (otherwise they run without it; the result is
  * the same fixed point).  The host waits after every map: it spins, unless the
  * device's scheduling flags ask for yielding or blocking waits, which it then
- * follows.  regc_reweight, regc_reweight2 and
+ * follows.  The library keeps up to 4 MB of page-locked host memory between
+ * solves (of all threads together), given back when the process ends.
+ * regc_reweight, regc_reweight2 and
  * regc_structure_reweight solve the same way; regc_mbar_last_info reports
  * what the last solve did. */
 REGC_API regc_status regc_mbar_solve(int S, const double *kT, const double *mu, double lambda0,

@@ -27,6 +27,8 @@
 
 #include <algorithm>
 #include <atomic>
+#include <chrono>
+#include <mutex>
 #include <type_traits>
 #include <vector>
 
@@ -1282,11 +1284,84 @@ struct SparseMat {
     }
 };
 
+// Page-locked memory of the solves, kept from one to the next: cudaFreeHost
+// waits for every stream of the device (a solve of 2 ms beside another stream's
+// kernel of 194 ms took 194 ms).  At most kKept bytes lie idle, in blocks of at
+// least kLeast, given back when the process ends; any thread takes any of them.
+class HostPool {
+public:
+    struct Block {
+        void* at = nullptr;
+        size_t bytes = 0;
+        unsigned long long mark = 0;   // as written to the block's first word
+    };
+    static HostPool& get() {
+        static HostPool pool;   // (made after the first CUDA call, so unmade before the runtime is)
+        return pool;
+    }
+    // A block of at least `bytes` behind its first 16; at = null: none to be had.
+    Block take(size_t bytes) {
+        bytes = std::max(bytes + 16, kLeast);
+        {
+            std::lock_guard<std::mutex> lock(mutex);
+            for (size_t k = 0; k < idle.size(); ++k) {
+                if (idle[k].bytes < bytes) continue;
+                const Block b = idle[k];
+                idle.erase(idle.begin() + k);
+                kept -= b.bytes;
+                if (alive(b)) return b;
+                --k;
+            }
+        }
+        Block b;
+        if (cudaHostAlloc(&b.at, bytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return Block{};
+        }
+        b.bytes = bytes;
+        b.mark = (unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count() ^
+                 (unsigned long long)reinterpret_cast<uintptr_t>(b.at) << 1 ^ 0x9e3779b97f4a7c15ull;
+        *static_cast<unsigned long long*>(b.at) = b.mark;
+        return b;
+    }
+    void give(const Block& b) {
+        if (!b.at) return;
+        {
+            std::lock_guard<std::mutex> lock(mutex);
+            if (kept + b.bytes <= kKept) {
+                idle.push_back(b);
+                kept += b.bytes;
+                return;
+            }
+        }
+        cudaFreeHost(b.at);
+    }
+    ~HostPool() {
+        for (const Block& b : idle)
+            if (alive(b)) cudaFreeHost(b.at);
+    }
+
+private:
+    static constexpr size_t kLeast = size_t(64) << 10, kKept = size_t(4) << 20;
+    // false after a reset of the device, which frees what its process had
+    static bool alive(const Block& b) {
+        cudaPointerAttributes a{};
+        if (cudaPointerGetAttributes(&a, b.at) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return false;
+        }
+        return a.type == cudaMemoryTypeHost && *static_cast<const unsigned long long*>(b.at) == b.mark;
+    }
+    std::mutex mutex;
+    std::vector<Block> idle;
+    size_t kept = 0;
+};
+
 // The host's side of the iteration: the weights it sends and the f_new it
 // reads, page-locked so that a map costs one asynchronous copy in and none
 // out.
 struct HostBlock {
-    void* block = nullptr;
+    HostPool::Block block;
     double *w = nullptr, *g = nullptr;
     unsigned long long* t = nullptr;
     int* empty = nullptr;
@@ -1297,12 +1372,9 @@ struct HostBlock {
         if (cudaGetDeviceFlags(&flags) != cudaSuccess) (void)cudaGetLastError();
         flags &= cudaDeviceScheduleMask;
         spin = flags != cudaDeviceScheduleYield && flags != cudaDeviceScheduleBlockingSync;
-        if (cudaHostAlloc(&block, size_t(2 * S + 4) * sizeof(double), cudaHostAllocDefault) != cudaSuccess) {
-            block = nullptr;
-            (void)cudaGetLastError();
-            return false;
-        }
-        w = static_cast<double*>(block);
+        block = HostPool::get().take((2 * size_t(S) + 4) * sizeof(double));
+        if (!block.at) return false;
+        w = static_cast<double*>(block.at) + 2;   // behind the block's mark
         g = w + S;
         t = reinterpret_cast<unsigned long long*>(g + S);
         empty = reinterpret_cast<int*>(t + 2);
@@ -1326,9 +1398,9 @@ struct HostBlock {
     }
     cudaStream_t s = nullptr;
     ~HostBlock() {
-        if (!block) return;
+        if (!block.at) return;
         cudaStreamSynchronize(s);   // (an early return may leave a map in flight)
-        cudaFreeHost(block);
+        HostPool::get().give(block);
     }
 };
 

@@ -4,6 +4,7 @@ import ctypes
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -111,3 +112,29 @@ def test_the_waits_follow_the_scheduling_flags():
     assert r.returncode == 0, r.stderr[-2000:]
     wall, cpu = (float(v) for v in r.stdout.split())
     assert cpu < 0.5 * wall
+
+
+def test_a_solve_does_not_wait_for_other_streams():
+    """After a first solve, solves (of more states, and of a thread of their own) end
+    while another stream still runs a kernel of some 0.2 s."""
+    torch = pytest.importorskip("torch")
+    small, large = close_states(64, 2000, seed=2), close_states(1024, 2000, seed=3)
+    mine, other = torch.cuda.Stream(), torch.cuda.Stream()
+
+    def solve(a):
+        mbar_solve(*a[:2], 1.0, *a[2:], tol=1e-300, max_iter=20, stream=mine)
+
+    solve(small)
+    thread = threading.Thread(target=lambda: (solve(small), solve(large)))
+    torch.cuda.synchronize()
+    with torch.cuda.stream(other):
+        torch.cuda._sleep(400_000_000)
+        end = torch.cuda.Event()
+        end.record(other)
+    solve(small)
+    solve(large)
+    thread.start()
+    thread.join()
+    running = not end.query()
+    torch.cuda.synchronize()
+    assert running
