@@ -736,18 +736,22 @@ __global__ void __launch_bounds__(256) sp_screen_kernel(const __grid_constant__ 
 // scanning every state took 3.5 times as long on 1024 states: each warp paid
 // for the union of its 32 bins' states and wrote 32 separate rows.)  What bounds
 // it is FP64; t_sb is therefore kept in the row between the two passes: 114
-// million entries 6.16 -> 5.5 ms.
-constexpr int kRowWarps = 8;
-template <bool TWO>
-__global__ void __launch_bounds__(32 * kRowWarps) sp_rows_kernel(const __grid_constant__ MbarDev m, SpDev p) {
-    const long long b = (long long)blockIdx.x * kRowWarps + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (b >= m.B) return;
+// million entries 6.16 -> 5.5 ms.  Short rows (short_rows) take kShortLanes lanes
+// each, eight bins a warp, since a whole warp is mostly idle on them: builds of 1,
+// 4, 16 states over 1e6 bins with a warp each / so 2.65 / 0.45, 2.66 / 0.47, 3.03 /
+// 1.23 ms (a thread per bin: 1.64, 2.50, 3.82).
+constexpr int kRowThreads = 256, kShortLanes = 4;
+template <bool TWO, int LANES>
+__global__ void __launch_bounds__(kRowThreads) sp_rows_kernel(const __grid_constant__ MbarDev m, SpDev p) {
+    const long long at_b = ((long long)blockIdx.x * kRowThreads + threadIdx.x) / LANES;
+    const int lane = threadIdx.x % LANES;
+    const bool act = at_b < m.B;
+    const long long b = act ? at_b : 0;
     const double E = m.E_b[b], N = (double)m.N_b[b], N2 = TWO ? (double)m.N2_b[b] : 0.0;
     const long long r0 = p.rp[b];
-    const int n = (int)(p.rp[b + 1] - r0);
+    const int n = act ? (int)(p.rp[b + 1] - r0) : 0;
     int* ci = p.ci + r0;
-    for (int w = lane; w < p.words; w += 32) {
+    for (int w = lane; act && w < p.words; w += LANES) {
         const size_t at = size_t(w) * m.B + b;
         int o = (int)p.pref[at];
         for (uint32_t bits = p.mask[at]; bits; bits &= bits - 1u) ci[o++] = 32 * w + __ffs(bits) - 1;
@@ -755,16 +759,16 @@ __global__ void __launch_bounds__(32 * kRowWarps) sp_rows_kernel(const __grid_co
     __syncwarp();
     double* cv = p.cv + r0;
     double M = -INFINITY;
-    for (int e = lane; e < n; e += 32) {
+    for (int e = lane; e < n; e += LANES) {
         const int s = ci[e];
         const double t = p.gs[s] - u_of<TWO>(m.a[s], m.c[s], TWO ? m.c2[s] : 0.0, E, N, N2);
         cv[e] = t;   // (read back by this lane: cheaper than taking it again in FP64)
         M = fmax(M, t);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
-    for (int e = lane; e < n; e += 32) cv[e] = exp(cv[e] - M);
-    if (lane == 0) {
+    for (int o = LANES / 2; o > 0; o >>= 1) M = fmax(M, __shfl_xor_sync(0xffffffffu, M, o));
+    for (int e = lane; e < n; e += LANES) cv[e] = exp(cv[e] - M);
+    if (act && lane == 0) {
         p.M[b] = M;
         p.H[b] = exp(m.lnH[b]);
     }
@@ -829,9 +833,14 @@ constexpr int kDLanes = 4;
 constexpr int kDThreads = 64;
 //
 // What bounds a small problem is the latency of a lane's entries one after the
-// other: eight are requested at a time, the next eight before these are added
-// (2040 bins of 125 entries: 23 us a map with both products, 13 us so).
-template <bool FINAL, class Weights>
+// other: AHEAD are requested at a time, the next AHEAD before these are added
+// (2040 bins of 125 entries: 23 us a map with both products, 13 us with eight).
+// Where rows are short (short_rows) eight requests are mostly beyond the row's
+// end, and what is spent on them counts: two there.  A map with 2 / 8 requests,
+// 1e6 bins: 1 state 130 / 176 us, 4 132 / 179, 16 164 / 196, 24 195 / 210, 32
+// 229 / 228, 64 349 / 347, 160 704 / 698 (one entry at a time, two chains: 131,
+// 128, 178, 267, 243, 411, 895).
+template <bool FINAL, class Weights, int AHEAD>
 __global__ void __launch_bounds__(kDThreads) sp_d_kernel(const __grid_constant__ MbarDev m,
                                                          const __grid_constant__ SpDev p,
                                                          const __grid_constant__ Weights wts) {
@@ -851,7 +860,7 @@ __global__ void __launch_bounds__(kDThreads) sp_d_kernel(const __grid_constant__
         const int n = (int)((p.rp[b + 1] - r0 + kDLanes - 1) / kDLanes);   // this lane's entries
         const int* ci = p.ci + r0;
         const double* cv = p.cv + r0;
-        constexpr int kU = 8;
+        constexpr int kU = AHEAD;   // even: the parity of an entry decides its chain
         int c[kU];
         double v[kU];
         auto request = [&](int k0) {
@@ -1124,6 +1133,10 @@ struct SparseMat {
     long long cap = 0, nnz = 0, pc_cap = 0, n_pieces = 0;
     size_t budget = 0;         // bytes left for the entries: half the memory free at the start less `fixed`
     int sms = 152;
+    // rows of fewer than kShortRow entries on average: where the two forms of
+    // the by-bin kernels take equally long (sp_d_kernel)
+    static constexpr int kShortRow = 32;
+    bool short_rows = false;
     std::vector<long long> h_begin;   // pc_begin and pc_state, pc_first as last uploaded
     std::vector<int> h_index;
     long long* tmp = nullptr;  // scan scratch
@@ -1233,7 +1246,13 @@ struct SparseMat {
             p.bi = p.ci + cap;
         }
         nnz = n_h;
-        sp_rows_kernel<TWO><<<(unsigned)((B + kRowWarps - 1) / kRowWarps), 32 * kRowWarps, 0, s>>>(m, p);
+        short_rows = nnz < (long long)kShortRow * B;
+        if (short_rows)
+            sp_rows_kernel<TWO, kShortLanes>
+                <<<(unsigned)(((long long)B * kShortLanes + kRowThreads - 1) / kRowThreads), kRowThreads, 0, s>>>(m, p);
+        else
+            sp_rows_kernel<TWO, 32><<<(unsigned)(((long long)B * 32 + kRowThreads - 1) / kRowThreads), kRowThreads, 0,
+                                      s>>>(m, p);
         sp_cols_kernel<false><<<cgrid, 256, 0, s>>>(m, p);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -1405,20 +1424,22 @@ struct HostBlock {
 };
 
 // The product d with the weights w (host, page-locked): with the launch where
-// they fit, else copied before it.
-template <bool FINAL>
+// they fit, else copied before it.  (Any number of bins: with the launch / by a
+// copy a map of 160 states takes 14.3 / 16.1 us on 2040 bins, of 448 states 126 /
+// 131 on 5e4 and 396 / 394 on 2e5, of 400 states 1602 / 1569 on 1e6.)
+template <bool FINAL, int AHEAD>
 cudaError_t launch_sp_d(const MbarDev& m, const SpDev& p, const double* w, cudaStream_t s) {
     const unsigned grid = (unsigned)((m.B * (long long)kDLanes + kDThreads - 1) / kDThreads);
     if (m.S <= kSmallS) {
         WeightsIn in;
         std::copy(w, w + m.S, in.w);
         std::fill(in.w + m.S, in.w + kSmallS, 0.0);
-        sp_d_kernel<FINAL, WeightsIn><<<grid, kDThreads, 0, s>>>(m, p, in);
+        sp_d_kernel<FINAL, WeightsIn, AHEAD><<<grid, kDThreads, 0, s>>>(m, p, in);
     } else {
         const cudaError_t e =
             cudaMemcpyAsync(p.w, w, size_t(m.S) * sizeof(double), cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return e;
-        sp_d_kernel<FINAL, NoWeights><<<grid, kDThreads, 0, s>>>(m, p, NoWeights{});
+        sp_d_kernel<FINAL, NoWeights, AHEAD><<<grid, kDThreads, 0, s>>>(m, p, NoWeights{});
     }
     return cudaGetLastError();
 }
@@ -1570,7 +1591,7 @@ cudaError_t mbar_solve_dev(const MbarDev& m, double tol, int max_iter, int* iter
         if (use_sp) {
             for (int k = 0; k < S; ++k) host.w[k] = exp(x[k] - fref_h[k]);
             *host.empty = 0;
-            err = launch_sp_d<false>(m, sp.p, host.w, s);
+            err = sp.short_rows ? launch_sp_d<false, 2>(m, sp.p, host.w, s) : launch_sp_d<false, 8>(m, sp.p, host.w, s);
             if (err != cudaSuccess) return err;
             sp_fp_kernel<<<(unsigned)sp.n_pieces, kFThreads, 0, s>>>(m, sp.p, ++map_no);
             err = cudaGetLastError();
@@ -1696,7 +1717,7 @@ cudaError_t mbar_solve_dev(const MbarDev& m, double tol, int max_iter, int* iter
     // D_b of the final f: on the matrix while it holds for f, else log-sum-exps
     if (use_sp && spread_of(x, fref_h) <= kSpreadAcc) {
         for (int k = 0; k < S; ++k) host.w[k] = exp(x[k] - fref_h[k]);
-        err = launch_sp_d<true>(m, sp.p, host.w, s);
+        err = sp.short_rows ? launch_sp_d<true, 2>(m, sp.p, host.w, s) : launch_sp_d<true, 8>(m, sp.p, host.w, s);
         if (err != cudaSuccess) return err;
     } else if (two) {
         d_kernel<true><<<dgrid128, 128, 0, s>>>(m, 1);
