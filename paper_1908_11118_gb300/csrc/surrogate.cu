@@ -750,16 +750,6 @@ __device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], const __nv_bfloat16* p
                  : "memory");
 }
 
-// 1 / d rounded to nearest, for 1 <= d < 2^117: the correction of a reciprocal
-// within one ulp by its exact residual (P. Markstein, IBM J. Res. Dev. 34,
-// 1990).  Equal to the division for each of those numbers (all of them were
-// compared), without its branch.
-__device__ __forceinline__ float reciprocal(float d) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-    return fmaf(r, fmaf(-d, r, 1.0f), r);
-}
-
 // z <- silu'(z) of a lane's 32 values, as dsilu_f.
 __device__ __forceinline__ void dsilu_all(float (&z)[2][4][4]) {
     bool far = false;
