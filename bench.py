@@ -15,7 +15,8 @@ own arm: device-timed (CUDA events on the library's stream) steps, with the L2
 flushed (256 MB memset) before every timed step; the JSON line adds the
 FP32-ALU roofline of the sweep kernel, the end-to-end rate through the C ABI
 with host buffers, sampled SM clocks, and the FP64 CPU oracle timed on a
-bounded sample on the host cores.
+bounded sample on the host cores.  The tables of the other workloads go to
+stderr, as one JSON line {"arms": ...}.
 reference arm: the FP64 CPU oracle on the same workload and metric.
 Under torchrun (N > 1) every rank runs its own independent 1024-replica grid
 (seed = rank): weak scaling, no collective on the data path.
@@ -93,6 +94,21 @@ def parse_args(argv=None):
     ap.add_argument("--da-steps-small", type=int, default=1000)
     ap.add_argument("--da-steps-large", type=int, default=60)
     return ap.parse_args(argv)
+
+
+# what the other arms measured: not part of the headline line
+ARMS = ("surrogate_da", "batched_uneven", "regcmd", "cluster_in_gas", "paper_lj_cycle", "production_phase_map",
+        "two_species", "cluster_production")
+
+
+def print_line(line):
+    """The headline as the one JSON line of stdout, short enough to be read whole
+    from the end of a log; the other arms' measurements (tables of some 30 kB) as
+    one JSON line {"arms": ...} on stderr."""
+    arms = {k: line[k] for k in ARMS if line.get(k) is not None}
+    if arms:
+        print(json.dumps({"arms": arms}), file=sys.stderr, flush=True)
+    print(json.dumps({k: v for k, v in line.items() if k not in ARMS}), flush=True)
 
 
 def dist_env():
@@ -1117,7 +1133,7 @@ def run_own(args):
             "two_species": two,
             "cluster_production": cluster_prod,
         }
-        print(json.dumps(line), flush=True)
+        print_line(line)
     g.close()
     if world > 1:
         torch.distributed.destroy_process_group()
