@@ -55,5 +55,7 @@ def test_exponential(differences, what):
 
 
 def test_a_difference_is_counted(differences):
-    """Beyond the range in use 2^-x is a subnormal number, which the short form drops."""
-    assert differences(4, 127.0, 140.0) > 10 ** 6
+    """Beyond the range in use 2^-x is a subnormal number, which the short form drops:
+    every argument from 127 to 140 differs."""
+    lo, hi = np.array([127.0, 140.0], np.float32).view(np.int32)
+    assert differences(4, 127.0, 140.0) == hi - lo
