@@ -836,10 +836,11 @@ constexpr int kDThreads = 64;
 // other: AHEAD are requested at a time, the next AHEAD before these are added
 // (2040 bins of 125 entries: 23 us a map with both products, 13 us with eight).
 // Where rows are short (short_rows) eight requests are mostly beyond the row's
-// end, and what is spent on them counts: two there.  A map with 2 / 8 requests,
-// 1e6 bins: 1 state 130 / 176 us, 4 132 / 179, 16 164 / 196, 24 195 / 210, 32
-// 229 / 228, 64 349 / 347, 160 704 / 698 (one entry at a time, two chains: 131,
-// 128, 178, 267, 243, 411, 895).
+// end, and what is spent on them counts as soon as the SMs are full: two there.  A
+// map with 2 / 8 requests, 1e6 bins: 1 state 130 / 176 us, 4 132 / 179, 16 164 /
+// 196, 24 195 / 210, 32 229 / 228, 64 349 / 347, 160 704 / 698 (one entry at a
+// time, two chains: 131, 128, 178, 267, 243, 411, 895); 28 states on 2e4 bins 16.7 /
+// 16.8, 5000 13.0 / 12.9, 2000 11.0 / 10.7, 500 9.6 / 9.3.
 template <bool FINAL, class Weights, int AHEAD>
 __global__ void __launch_bounds__(kDThreads) sp_d_kernel(const __grid_constant__ MbarDev m,
                                                          const __grid_constant__ SpDev p,
@@ -1133,8 +1134,10 @@ struct SparseMat {
     long long cap = 0, nnz = 0, pc_cap = 0, n_pieces = 0;
     size_t budget = 0;         // bytes left for the entries: half the memory free at the start less `fixed`
     int sms = 152;
-    // rows of fewer than kShortRow entries on average: where the two forms of
-    // the by-bin kernels take equally long (sp_d_kernel)
+    // rows of fewer than kShortRow entries on average, and so many bins that the
+    // SMs are full (two CTAs of sp_d_kernel an SM): where the two forms of the
+    // by-bin kernels take equally long (sp_d_kernel; a build of 36 states over 360
+    // bins 95 us with four lanes a row, 89 with a warp)
     static constexpr int kShortRow = 32;
     bool short_rows = false;
     std::vector<long long> h_begin;   // pc_begin and pc_state, pc_first as last uploaded
@@ -1246,7 +1249,7 @@ struct SparseMat {
             p.bi = p.ci + cap;
         }
         nnz = n_h;
-        short_rows = nnz < (long long)kShortRow * B;
+        short_rows = nnz < (long long)kShortRow * B && (long long)kDLanes * B >= 2LL * sms * kDThreads;
         if (short_rows)
             sp_rows_kernel<TWO, kShortLanes>
                 <<<(unsigned)(((long long)B * kShortLanes + kRowThreads - 1) / kRowThreads), kRowThreads, 0, s>>>(m, p);
