@@ -1132,7 +1132,7 @@ struct SparseMat {
     void* entries = nullptr;   // cap entries: cv, bv (double), ci, bi (int)
     void* pieces = nullptr;    // pc_begin, pc_sum, pc_state, pc_first for up to pc_cap pieces
     long long cap = 0, nnz = 0, pc_cap = 0, n_pieces = 0;
-    size_t budget = 0;         // bytes left for the entries: half the memory free at the start less `fixed`
+    size_t fixed_bytes = 0;
     int sms = 152;
     // rows of fewer than kShortRow entries on average, and so many bins that the
     // SMs are full (two CTAs of sp_d_kernel an SM): where the two forms of the
@@ -1152,7 +1152,8 @@ struct SparseMat {
     }
 
     // cudaErrorMemoryAllocation where the masks alone pass half the free device
-    // memory (nothing is allocated then).
+    // memory (nothing is allocated then; asked where they are no trifle, since the
+    // question takes as long as a map of a small problem).
     cudaError_t init(const MbarDev& m) {
         const size_t B = size_t(m.B), S = size_t(m.S);
         int dev = 0;
@@ -1171,13 +1172,15 @@ struct SparseMat {
         const size_t SC = S * p.n_chunk, words = size_t(p.words) * B;
         const size_t nt = std::max((B + kScanChunk - 1) / kScanChunk, (SC + kScanChunk - 1) / kScanChunk) + 1;
         const size_t n8 = (B + 1) + (SC + 1) + 3 * B + 3 * S + nt;
-        const size_t bytes = n8 * 8 + words * 8 + (S + 1) * 4;
-        size_t fr = 0, tot = 0;
-        cudaError_t e = cudaMemGetInfo(&fr, &tot);
-        if (e != cudaSuccess) return e;
-        if (bytes > fr / 2) return cudaErrorMemoryAllocation;
-        budget = fr / 2 - bytes;
-        e = cudaMallocAsync(&fixed, bytes, s);
+        fixed_bytes = n8 * 8 + words * 8 + (S + 1) * 4;
+        cudaError_t e = cudaSuccess;
+        if (fixed_bytes > (size_t(16) << 20)) {
+            size_t fr = 0, tot = 0;
+            e = cudaMemGetInfo(&fr, &tot);
+            if (e == cudaSuccess && fixed_bytes > fr / 2) e = cudaErrorMemoryAllocation;
+            if (e != cudaSuccess) return e;
+        }
+        e = cudaMallocAsync(&fixed, fixed_bytes, s);
         if (e != cudaSuccess) {
             fixed = nullptr;
             return e;
@@ -1236,7 +1239,7 @@ struct SparseMat {
             e = cudaMemGetInfo(&fr, &tot);
             if (e != cudaSuccess) return e;
             const size_t need = size_t(n_h) * 24;
-            if (need > fr / 2 || need > budget) return cudaSuccess;
+            if (need + fixed_bytes > (fr + fixed_bytes) / 2) return cudaSuccess;
             if (cudaMallocAsync(&entries, need, s) != cudaSuccess) {
                 entries = nullptr;
                 (void)cudaGetLastError();   // out of memory is not sticky
