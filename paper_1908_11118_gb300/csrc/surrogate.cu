@@ -334,27 +334,6 @@ __device__ __forceinline__ float sum_over_g(float v) {
     return v;
 }
 
-// Write parameter i of the master vector into the operand copies.
-__device__ __forceinline__ void tc_store_param(TcSmem& sm, int i, float v) {
-    constexpr int o1 = kNF * kNH, o2 = o1 + kNH, o3 = o2 + kNH * kNH, o4 = o3 + kNH, o5 = o4 + kNH;
-    if (i < o1) {
-        sm.w1u[i % kNH][i / kNH] = __float2bfloat16_rn(v);   // W1[k][u]
-    } else if (i < o2) {
-        sm.b1[i - o1] = v;
-    } else if (i < o3) {
-        const int u = (i - o2) / kNH, q = (i - o2) % kNH;    // W2[u][q]
-        const __nv_bfloat16 w = __float2bfloat16_rn(v);
-        sm.w2r[u][q] = w;
-        sm.w2u[q][u] = w;
-    } else if (i < o4) {
-        sm.b2[i - o3] = v;
-    } else if (i < o5) {
-        sm.w3[i - o4] = v;
-    } else {
-        sm.b3 = v;
-    }
-}
-
 // Layer-1 A registers of one row (h = 0: row g, 1: row g + 8 of 16-row tile mt
 // of this warp) from its features 2t, 2t + 1 (lo) and 2t + 8, 2t + 9 (hi), and
 // the row's place in the transposed copy.
@@ -632,7 +611,26 @@ __global__ void __launch_bounds__(kTcRows) grad_tc_kernel(const float* theta, co
     TcSmem& sm = *reinterpret_cast<TcSmem*>(tc_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, t = lane & 3;
-    for (int i = tid; i < kNParams; i += kTcRows) tc_store_param(sm, i, theta[i]);
+    // the operand copies of the masters, array by array (looking up the place of each
+    // of the 5313 parameters: ten steps of 1025 rows 528 us instead of 463)
+    const float* W1 = theta;
+    const float* B1 = W1 + kNF * kNH;
+    const float* W2 = B1 + kNH;
+    const float* B2 = W2 + kNH * kNH;
+    const float* W3 = B2 + kNH;
+    for (int i = tid; i < kNH * kNH; i += kTcRows) {
+        const int u = i / kNH, v = i % kNH;   // W2[u][v]
+        const __nv_bfloat16 w = __float2bfloat16_rn(W2[i]);
+        sm.w2r[u][v] = w;
+        sm.w2u[v][u] = w;
+        if (i < kNF * kNH) sm.w1u[i % kNH][i / kNH] = __float2bfloat16_rn(W1[i]);   // W1[k][u]
+        if (i < kNH) {
+            sm.w3[i] = W3[i];
+            sm.b1[i] = B1[i];
+            sm.b2[i] = B2[i];
+        }
+    }
+    if (tid == 0) sm.b3 = W3[kNH];
     // layer-1 A fragments: this warp's rows 32 warp + 16 mt + (g, g + 8)
     const int row0 = blockIdx.x * kTcRows + warp * 32;
     uint32_t ax[2][4];
