@@ -1134,10 +1134,13 @@ struct SparseMat {
     long long cap = 0, nnz = 0, pc_cap = 0, n_pieces = 0;
     size_t fixed_bytes = 0;
     int sms = 152;
-    // rows of fewer than kShortRow entries on average, and so many bins that the
-    // SMs are full (two CTAs of sp_d_kernel an SM): where the two forms of the
-    // by-bin kernels take equally long (sp_d_kernel; a build of 36 states over 360
-    // bins 95 us with four lanes a row, 89 with a warp)
+    // fewer than kShortRow states, so no row is longer, and so many bins that the
+    // SMs are full (two CTAs of sp_d_kernel an SM): where the two forms of the by-bin
+    // kernels take equally long (sp_d_kernel; a build of 36 states over 360 bins 95 us
+    // with four lanes a row, 89 with a warp).  Rows of many states can be short on
+    // average and have long ones among them: three builds of 60284 bins and 1024
+    // states with fewer than 32 entries a row on average took 1.04 ms with four lanes
+    // a row, 0.55 with a warp.
     static constexpr int kShortRow = 32;
     bool short_rows = false;
     std::vector<long long> h_begin;   // pc_begin and pc_state, pc_first as last uploaded
@@ -1163,6 +1166,7 @@ struct SparseMat {
             sms = 152;
         }
         p.words = (m.S + 31) / 32;
+        short_rows = m.S < kShortRow && (long long)kDLanes * m.B >= 2LL * sms * kDThreads;
         // bins per chunk of the by-state order: 1024, fewer where the chunks
         // times the words would not give every SM some 32 warps
         const size_t tiles = (B + 31) / 32;
@@ -1252,7 +1256,6 @@ struct SparseMat {
             p.bi = p.ci + cap;
         }
         nnz = n_h;
-        short_rows = nnz < (long long)kShortRow * B && (long long)kDLanes * B >= 2LL * sms * kDThreads;
         if (short_rows)
             sp_rows_kernel<TWO, kShortLanes>
                 <<<(unsigned)(((long long)B * kShortLanes + kRowThreads - 1) / kRowThreads), kRowThreads, 0, s>>>(m, p);
