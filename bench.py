@@ -45,9 +45,9 @@ import workloads as W  # noqa: E402
 SWEEPS_PER_STEP = 10
 # DRAM bytes (read + write) of one sweep-kernel launch on the benchmark
 # workload from an ncu capture of the current kernel
-# (dram__bytes_read.sum 4336384 + dram__bytes_write.sum 0); None whenever the
+# (dram__bytes_read.sum 4544256 + dram__bytes_write.sum 0); None whenever the
 # kernel has changed since its last capture
-SWEEP_TRAFFIC_BYTES = 4336384 + 0
+SWEEP_TRAFFIC_BYTES = 4544256 + 0
 FLOPS_PER_PAIR = 20            # dx,dy,dz 3, xy minimum image 4, r^2 5, r^-2 1, s^6 3, 4eps s^6(s^6-1) 4
 SM_COUNT, FP32_LANES, MAX_SM_MHZ = 152, 128, 2070.0
 METRIC = "GCMC trial moves/s over all replicas"

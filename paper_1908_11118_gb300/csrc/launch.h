@@ -17,6 +17,14 @@ namespace regc {
 //   periodic cube, 125 cells, 16 walkers:   160 / 165 at 68, 164 / 172 at 96, 178 / 176 at 128
 //   periodic cube, 4096 walkers (27 per SM):   416 / 544 at 68, 475 / 551 at 128, 533 / 564 at 160, 593 / 583 at 192
 //   A18, 40 cells, 160 walkers of 20 particles:   78 / 101
+// Above kDirectMax every walker has cells, also in boxes of few cells, where the
+// direct form would still be the faster one (N nearly Nmax, four and one warps):
+//   A18, 40 cells, 160 walkers:   109 / 133 at 192, 125 / 143 at 256, 133 / 153 at 320
+//   fcc(100), at most 27 cells, 16 and 4096 walkers:   175 / 255 and 780 / 1438 at 192
+// Where that ends was not measured; a line beyond it is a change of its own.  The
+// rule goes by Nmax, which is known when the shared memory is laid out; the cost goes
+// by N, so a walker that stays far below a large Nmax keeps its cells although all
+// its particles would cost less.
 constexpr int kDirectMax = 160;
 
 inline int direct_limit(int ncell, long long walkers, int sms) {
