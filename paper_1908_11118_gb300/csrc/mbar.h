@@ -54,7 +54,7 @@ MbarInfo mbar_last_info();
 
 // Solve the self-consistent equations from f = 0 (the plain fixed-point map
 // with Anderson acceleration) until max |G(f) - f| < tol or max_iter maps.
-// Synchronises the stream after every map.
+// The host waits for every map.
 // With allow_matrix (and every state sampled) the iterations run on the
 // kept entries of the kernel matrix K_sb = exp(-u_s(b) + ln Omega_s + f_ref,s
 // - max_k(...)) (those within e^-70 of their bin's largest), allocated on the

@@ -138,3 +138,50 @@ def test_a_solve_does_not_wait_for_other_streams():
     running = not end.query()
     torch.cuda.synchronize()
     assert running
+
+
+def test_threads_share_the_page_locked_memory():
+    """Solves of different sizes in eight threads at once equal the same solves alone."""
+    problems = [close_states(S, 500 + S, seed=S) for S in (1, 30, 64, 300, 449, 700, 1024, 5000)]
+
+    def solve(a):
+        return mbar_solve(*a[:2], 1.0, *a[2:], tol=1e-11)
+
+    alone = [solve(a) for a in problems]
+    got = [[None] * len(problems) for _ in range(3)]
+
+    def work(k):
+        for turn in got:
+            turn[k] = solve(problems[k])
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(len(problems))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for turn in got:
+        for (f, D, it), (g, E, jt) in zip(alone, turn):
+            assert np.array_equal(f, g) and np.array_equal(D, E) and it == jt
+
+
+RESET = """
+import ctypes
+import numpy as np
+from paper_1908_11118_gb300 import mbar_solve
+rng = np.random.default_rng(0)
+S, B = 64, 2000
+N = np.sort(rng.integers(0, 25, B))
+E, H = -2.0 * N + rng.normal(size=B), rng.uniform(1.0, 5.0, B)
+a = (np.linspace(0.9, 1.4, S), np.linspace(-4.0, -3.0, S), 1.0, np.full(S, H.sum() / S), N, E, H)
+first = mbar_solve(*a)
+assert ctypes.CDLL("libcuda.so.1").cuDevicePrimaryCtxReset_v2(0) == 0     # this process's own context
+again = mbar_solve(*a)
+assert np.array_equal(first[0], again[0]) and np.array_equal(first[1], again[1])
+"""
+
+
+def test_a_solve_after_the_context_was_reset():
+    """The page-locked memory kept from a solve goes with its context."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", RESET], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
